@@ -4,6 +4,7 @@
 // canonical <-> GEMM weight layouts. All reductions run in a fixed order.
 #include <algorithm>
 
+#include "lstm_cell.cuh"
 #include "nn_kernels.cuh"
 
 namespace ddppo {
@@ -645,8 +646,6 @@ int launch_colsum2(const float* in0, const float* in1, int R, int Cc, int ld, fl
 }
 
 // ---------------------------------------------------------------- LSTM cell
-__device__ __forceinline__ float sigm(float x) { return 1.0f / (1.0f + expf(-x)); }
-
 __global__ void lstm_fwd_kernel(LstmStep a) {
   DDPPO_PDL_ENTRY();
   const size_t total = (size_t)a.E * a.H;
@@ -659,10 +658,9 @@ __global__ void lstm_fwd_kernel(LstmStep a) {
     const float zf = a.gx[gb + a.H + j] + a.gh[gb + a.H + j];
     const float zg = a.gx[gb + 2 * a.H + j] + a.gh[gb + 2 * a.H + j];
     const float zo = a.gx[gb + 3 * a.H + j] + a.gh[gb + 3 * a.H + j];
-    const float i = sigm(zi), f = sigm(zf), g = tanhf(zg), o = sigm(zo);
     const float cp = a.m[e] ? a.c_prev[idx] : 0.f;
-    const float c = f * cp + i * g;
-    const float h = o * tanhf(c);
+    float i, f, g, o, c, h;
+    lstm_cell_fwd(zi, zf, zg, zo, cp, i, f, g, o, c, h);
     a.gates[gb + j] = i; a.gates[gb + a.H + j] = f;
     a.gates[gb + 2 * a.H + j] = g; a.gates[gb + 3 * a.H + j] = o;
     a.c[idx] = c;
@@ -714,14 +712,9 @@ __global__ void lstm_bwd_kernel(LstmBack a) {
     const bool carry = a.m_next && a.m_next[e];
     float dh = a.dh_above[idx];
     if (carry && a.dh_rec) dh += a.dh_rec[idx];
-    const float tc = tanhf(c);
-    float dc = dh * o * (1.f - tc * tc);
-    if (carry) dc += a.dc_carry[idx];
-    const float dzi = dc * g * i * (1.f - i);
-    const float dzf = dc * cp * f * (1.f - f);
-    const float dzg = dc * i * (1.f - g * g);
-    const float dzo = dh * tc * o * (1.f - o);
-    a.dc_carry[idx] = dc * f;
+    float dzi, dzf, dzg, dzo, dco;
+    lstm_cell_bwd(i, f, g, o, c, cp, dh, carry, carry ? a.dc_carry[idx] : 0.f, dzi, dzf, dzg, dzo, dco);
+    a.dc_carry[idx] = dco;
     a.dg32[gb + j] = dzi; a.dg32[gb + a.H + j] = dzf;
     a.dg32[gb + 2 * a.H + j] = dzg; a.dg32[gb + 3 * a.H + j] = dzo;
     if (a.dg_op) {
