@@ -236,8 +236,9 @@ static int alloc_f8(Net& n, int pool_hw) {
 static int alloc_encoder(Net& n) {
   const size_t NC = n.NC;
   auto conv_bufs = [&](ConvL& c) -> int {
+    // (the columns past k k cin stay zero: the preparation writes the others)
     DDPPO_TRY(nalloc_op(n, &c.wg, (size_t)c.cout * c.Kp));
-    DDPPO_TRY(nalloc_op(n, &c.wgT, (size_t)c.cout * c.Kp));
+    DDPPO_CHECK_CUDA(cudaMemset(c.wg, 0, (size_t)c.cout * c.Kp * esz(n)));
     DDPPO_TRY(nalloc(n, &c.dwg, (size_t)c.cout * c.Kp));
     DDPPO_TRY(nalloc(n, &c.z, NC * c.Ho * c.Wo * c.cout));
     // a stride-1 'same' convolution's input gradient is a convolution of its output
@@ -246,6 +247,9 @@ static int alloc_encoder(Net& n) {
     if (c.dgrad_as_conv) {
       DDPPO_TRY(nalloc_op(n, &c.wgR, (size_t)c.cin * c.k * c.k * c.cout));
       n.max_col = std::max(n.max_col, (size_t)c.H * c.W * c.k * c.k * c.cout);
+    } else {
+      DDPPO_TRY(nalloc_op(n, &c.wgT, (size_t)c.cout * c.Kp));
+      DDPPO_CHECK_CUDA(cudaMemset(c.wgT, 0, (size_t)c.cout * c.Kp * esz(n)));
     }
     n.max_col = std::max(n.max_col, (size_t)c.Ho * c.Wo * c.Kp);
     n.max_dz = std::max(n.max_dz, (size_t)c.Ho * c.Wo * c.cout);
@@ -422,14 +426,44 @@ static int init_params(Net& n, cudaStream_t s) {
   return DDPPO_OK;
 }
 
+// the table of the weights' operand copies (buffers and offsets are fixed at creation)
+static int build_weight_prep(Net& n) {
+  std::vector<WPrep> t;
+  std::vector<uint16_t> entry;
+  auto add = [&](WPrep e) {
+    e.first = (int)entry.size();
+    entry.insert(entry.end(), (size_t)weight_prep_blocks(e), (uint16_t)t.size());
+    t.push_back(e);
+  };
+  auto matrix = [](int64_t src, int rows, int cin, int kk, int ld, void* wg, void* wgT, void* wgR) {
+    WPrep e;
+    e.src = src; e.rows = rows; e.cin = cin; e.kk = kk; e.ld = ld;
+    e.wg = wg; e.wgT = wgT; e.wgR = wgR;
+    return e;
+  };
+  for (ConvL* c : n.convs)
+    add(matrix(c->w_off, c->cout, c->cin, c->k * c->k, c->Kp, c->wg, c->wgT, c->wgR));
+  if (n.F > 0) add(matrix(n.vis_w, n.H, n.featC, n.featHW, n.F, n.Wv, n.WvT, nullptr));
+  for (int l = 0; l < n.L; ++l) {
+    LstmL& q = n.lstm[l];
+    add(matrix(q.wih, 4 * n.H, q.In, 1, q.In, q.Wih, q.WihT, nullptr));
+    add(matrix(q.whh, 4 * n.H, n.H, 1, n.H, q.Whh, q.WhhT, nullptr));
+    WPrep e;
+    e.src = q.bih; e.src2 = q.bhh; e.rows = 4 * n.H; e.wg = q.bsum;
+    add(e);
+  }
+  n.wprep_blocks = (int)entry.size();
+  DDPPO_TRY(nalloc(n, &n.wprep, t.size()));
+  DDPPO_TRY(nalloc(n, &n.wprep_entry, entry.size()));
+  DDPPO_CHECK_CUDA(cudaMemcpy(n.wprep, t.data(), t.size() * sizeof(WPrep), cudaMemcpyHostToDevice));
+  DDPPO_CHECK_CUDA(cudaMemcpy(n.wprep_entry, entry.data(), entry.size() * sizeof(uint16_t),
+                              cudaMemcpyHostToDevice));
+  return DDPPO_OK;
+}
+
 // canonical fp32 params -> GEMM operands in the precision's dtype
 int net_prep_weights(Net& n, cudaStream_t s) {
-  for (ConvL* c : n.convs) {
-    DDPPO_TRY(launch_conv_w_prep(n.params + c->w_off, c->cout, c->cin, c->k, c->Kp, c->wg, c->wgT,
-                                 n.bf, s));
-    if (c->dgrad_as_conv)
-      DDPPO_TRY(launch_conv_w_flip(n.params + c->w_off, c->cout, c->cin, c->k, c->wgR, n.bf, s));
-  }
+  DDPPO_TRY(launch_weight_prep(n.wprep, n.wprep_entry, n.wprep_blocks, n.params, n.bf, s));
   for (SxL& X : n.sx)
     DDPPO_TRY(launch_gconv_w_prep(n.params + X.c2.w_off, X.c2.C, X.c2.cpg, X.c2.wg, n.bf, s));
   if (n.f8) {
@@ -442,17 +476,6 @@ int net_prep_weights(Net& n, cudaStream_t s) {
       DDPPO_TRY(launch_amax(c->wg, true, cnt, c->w8_amax, s));
       DDPPO_TRY(launch_quant_e4m3(c->wg, true, cnt, c->w8_amax, c->w8_scale, c->wg8, s));
     }
-  }
-  if (n.F > 0)
-    DDPPO_TRY(launch_vis_w_prep(n.params + n.vis_w, n.H, n.featC, n.featHW, n.Wv, n.WvT, n.bf, s));
-  for (int l = 0; l < n.L; ++l) {
-    LstmL& q = n.lstm[l];
-    const int G4 = 4 * n.H;
-    DDPPO_TRY(launch_cast(n.params + q.wih, q.Wih, n.bf, (size_t)G4 * q.In, s));
-    DDPPO_TRY(launch_transpose(n.params + q.wih, false, q.WihT, n.bf, G4, q.In, q.In, s));
-    DDPPO_TRY(launch_cast(n.params + q.whh, q.Whh, n.bf, (size_t)G4 * n.H, s));
-    DDPPO_TRY(launch_transpose(n.params + q.whh, false, q.WhhT, n.bf, G4, n.H, n.H, s));
-    DDPPO_TRY(launch_add_vec(n.params + q.bih, n.params + q.bhh, q.bsum, G4, s));
   }
   return DDPPO_OK;
 }
@@ -551,7 +574,9 @@ int net_create(ddppo_ctx* x) {
   DDPPO_TRY(nalloc(n, &n.adv_norm, (size_t)n.T * n.E));
   DDPPO_TRY(nalloc(n, &n.scal, 8));
   DDPPO_TRY(nalloc(n, &n.stats_tmp, 8 * 64));
-  DDPPO_TRY(nalloc(n, &n.norm, 1));
+  DDPPO_TRY(nalloc(n, &n.opt, 3));
+  DDPPO_TRY(nalloc(n, &n.opt_cnt, 1));
+  DDPPO_CHECK_CUDA(cudaMemset(n.opt_cnt, 0, sizeof(int)));
   DDPPO_TRY(nalloc(n, &n.act_h, (size_t)n.L * n.E * Hd));
   DDPPO_TRY(nalloc(n, &n.act_c, (size_t)n.L * n.E * Hd));
   DDPPO_TRY(nalloc(n, &n.post_done, n.E));
@@ -568,6 +593,7 @@ int net_create(ddppo_ctx* x) {
     DDPPO_CHECK_CUDA(cudaEventCreate(&n.timer.ev[i]));
     DDPPO_CHECK_CUDA(cudaEventCreate(&n.rc_timer.ev[i]));
   }
+  DDPPO_TRY(build_weight_prep(n));
   DDPPO_TRY(init_params(n, 0));
   DDPPO_TRY(net_prep_weights(n, 0));
   return DDPPO_OK;

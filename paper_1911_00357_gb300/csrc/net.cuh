@@ -17,7 +17,7 @@ struct ConvL {
   int Kp = 0;
   int H = 0, W = 0, Ho = 0, Wo = 0;
   void* wg = nullptr;   // [cout, Kp] op dtype
-  void* wgT = nullptr;  // [Kp, cout] op dtype (dgrad through col2im)
+  void* wgT = nullptr;  // [Kp, cout] op dtype (dgrad through col2im; null where dgrad_as_conv)
   void* wgR = nullptr;  // [cin, k*k*cout] op dtype: flipped, channel-swapped kernel (stride-1 dgrad)
   bool dgrad_as_conv = false;
   float* dwg = nullptr; // [cout, Kp] fp32 gradient in GEMM layout
@@ -125,6 +125,10 @@ struct Net {
   uint8_t* pool_arg = nullptr;
   BlockL blocks[8];
   std::vector<SxL> sx;                  // SE-ResNeXt bottlenecks (net_kind 3, 4)
+  // operand copies of the weights, all in one launch (device table; block -> entry)
+  WPrep* wprep = nullptr;
+  uint16_t* wprep_entry = nullptr;
+  int wprep_blocks = 0;
   float* gw_part = nullptr; size_t gw_part_elems = 0;  // grouped-conv weight-gradient partials
   float* se_dg = nullptr; float* se_dq = nullptr; float* se_dh = nullptr; float* se_dm = nullptr;
   ConvL cmp;
@@ -166,7 +170,9 @@ struct Net {
   uint8_t* masks_mb = nullptr; int32_t* act_mb = nullptr; float* logp_mb = nullptr;
   float* adv_mb = nullptr; float* ret_mb = nullptr; float* h0_mb = nullptr; float* c0_mb = nullptr;
   int32_t* perm = nullptr; float* adv_norm = nullptr; float* scal = nullptr;
-  float* stats_tmp = nullptr; float* norm = nullptr;
+  float* stats_tmp = nullptr;
+  float* opt = nullptr;    // [3] gradient norm, Adam's two bias corrections
+  int* opt_cnt = nullptr;  // blocks of the norm reduction that have finished (0 between launches)
   float* act_h = nullptr; float* act_c = nullptr;  // bootstrap state sink
 
   // last evaluate (inputs read again by backward)

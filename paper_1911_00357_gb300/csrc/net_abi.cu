@@ -223,11 +223,10 @@ static int update_body(ddppo_ctx* x, const ddppo_rollout* ro, const ddppo_ppo_hp
                                 hp->clip, hp->value_coef, hp->entropy_coef, st, n.dlogits,
                                 n.dvalues, n.scratch, n.scratch_elems, s));
       DDPPO_TRY(net_backward(n, n.dlogits, n.dvalues, s));
-      DDPPO_TRY(launch_grad_norm(n.grad, n.P, n.norm, n.scratch, n.scratch_elems, s));
-      DDPPO_TRY(launch_copy_scalar(st + 6, n.norm, s));
-      DDPPO_TRY(launch_adam(n.params, n.grad, n.adam_m, n.adam_v, n.P,
-                            hp->max_grad_norm > 0.f ? n.norm : nullptr, hp->max_grad_norm, hp->lr,
-                            hp->beta1, hp->beta2, hp->adam_eps, n.d_steps + 1, k + 1, s));
+      DDPPO_TRY(launch_opt_scalars(n.grad, 1.f, n.P, hp->beta1, hp->beta2, n.d_steps + 1, k + 1,
+                                   n.opt, st + 6, n.opt_cnt, n.scratch, n.scratch_elems, s));
+      DDPPO_TRY(launch_adam(n.params, n.grad, 1.f, n.adam_m, n.adam_v, n.P, n.opt,
+                            hp->max_grad_norm, hp->lr, hp->beta1, hp->beta2, hp->adam_eps, s));
       DDPPO_TRY(net_prep_weights(n, s));
     }
   }
@@ -235,14 +234,6 @@ static int update_body(ddppo_ctx* x, const ddppo_rollout* ro, const ddppo_ppo_hp
 }
 
 // ---- the update one minibatch at a time (gradients exchanged between workers, Eq. 4) ----
-__global__ void scale_copy_kernel(const float* __restrict__ g, float scale, float* __restrict__ out,
-                                  size_t n) {
-  DDPPO_PDL_ENTRY();
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x)
-    out[i] = scale * g[i];
-}
-
 extern "C" int ddppo_ppo_grad(ddppo_ctx* x, const ddppo_rollout* ro, const ddppo_ppo_hparams* hp,
                               int32_t T_valid, int32_t epoch, int32_t k, float* grad, float* stats,
                               void* stream) {
@@ -298,16 +289,10 @@ extern "C" int ddppo_apply_grad(ddppo_ctx* x, const float* grad, float scale,
   Net& n = *x->net;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t P = (size_t)n.P;
-  ::ddppo::launch_k(scale_copy_kernel, (unsigned)std::min<size_t>((P + 255) / 256, 4096), 256, 0, s, grad, scale,
-                                                                                     n.grad, P);
-  DDPPO_CHECK_LAUNCH();
-  DDPPO_TRY(launch_grad_norm(n.grad, P, n.norm, n.scratch, n.scratch_elems, s));
-  if (stats) DDPPO_TRY(launch_copy_scalar(stats + 6, n.norm, s));
-  ::ddppo::launch_k(set_steps_kernel, 1, 1, 0, s, n.d_steps, hp->update_index, n.adam_t);
-  DDPPO_CHECK_LAUNCH();
-  DDPPO_TRY(launch_adam(n.params, n.grad, n.adam_m, n.adam_v, P,
-                        hp->max_grad_norm > 0.f ? n.norm : nullptr, hp->max_grad_norm, hp->lr,
-                        hp->beta1, hp->beta2, hp->adam_eps, n.d_steps + 1, 1, s));
+  DDPPO_TRY(launch_opt_scalars(grad, scale, P, hp->beta1, hp->beta2, nullptr, n.adam_t + 1, n.opt,
+                               stats ? stats + 6 : nullptr, n.opt_cnt, n.scratch, n.scratch_elems, s));
+  DDPPO_TRY(launch_adam(n.params, grad, scale, n.adam_m, n.adam_v, P, n.opt, hp->max_grad_norm,
+                        hp->lr, hp->beta1, hp->beta2, hp->adam_eps, s));
   DDPPO_TRY(net_prep_weights(n, s));
   n.adam_t += 1;
   return DDPPO_OK;

@@ -347,40 +347,7 @@ int launch_col2im(const ConvGeom& g, const float* dcol, float* dx, bool accumula
   return DDPPO_OK;
 }
 
-// ---------------------------------------------------------------- transpose / cast
-template <typename Ti, typename To>
-__global__ void transpose_kernel(const Ti* __restrict__ in, To* __restrict__ out, int R, int Cc,
-                                 int ld_in) {
-  DDPPO_PDL_ENTRY();
-  __shared__ float tile[32][33];
-  const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;  // rows on x: R can be in the millions
-  for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-    const int r = r0 + j, c = c0 + threadIdx.x;
-    tile[j][threadIdx.x] = (r < R && c < Cc) ? to_f(in[(size_t)r * ld_in + c]) : 0.f;
-  }
-  __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-    const int c = c0 + j, r = r0 + threadIdx.x;
-    if (c < Cc && r < R) out[(size_t)c * R + r] = from_f<To>(tile[threadIdx.x][j]);
-  }
-}
-
-int launch_transpose(const void* in, bool in_bf16, void* out, bool out_bf16, int R, int Cc,
-                     int ld_in, cudaStream_t s) {
-  if (R == 0 || Cc == 0) return DDPPO_OK;
-  dim3 grid((R + 31) / 32, (Cc + 31) / 32), blk(32, 8);
-  if (in_bf16 && out_bf16)
-    ::ddppo::launch_k(transpose_kernel<__nv_bfloat16, __nv_bfloat16>, grid, blk, 0, s, (const __nv_bfloat16*)in, (__nv_bfloat16*)out, R, Cc, ld_in);
-  else if (in_bf16)
-    ::ddppo::launch_k(transpose_kernel<__nv_bfloat16, float>, grid, blk, 0, s, (const __nv_bfloat16*)in, (float*)out, R, Cc, ld_in);
-  else if (out_bf16)
-    ::ddppo::launch_k(transpose_kernel<float, __nv_bfloat16>, grid, blk, 0, s, (const float*)in, (__nv_bfloat16*)out, R, Cc, ld_in);
-  else
-    ::ddppo::launch_k(transpose_kernel<float, float>, grid, blk, 0, s, (const float*)in, (float*)out, R, Cc, ld_in);
-  DDPPO_CHECK_LAUNCH();
-  return DDPPO_OK;
-}
-
+// ---------------------------------------------------------------- cast
 __global__ void cast_kernel(const float* __restrict__ in, void* out, int bf, size_t n) {
   DDPPO_PDL_ENTRY();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -978,50 +945,6 @@ int launch_gather_rows(const void* in, void* out, const int32_t* idx, int T, int
 }
 
 // ---------------------------------------------------------------- weight layouts
-// canonical w[co, ci, ky, kx] -> wg[co, (ky*k + kx)*cin + ci] and wgT[(..), co]; pad zero
-__global__ void conv_w_prep_kernel(const float* __restrict__ w, int cout, int cin, int k, int Kp,
-                                   void* wg, void* wgT, int bf) {
-  DDPPO_PDL_ENTRY();
-  const size_t total = (size_t)cout * Kp;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (size_t)gridDim.x * blockDim.x) {
-    const int co = (int)(idx / Kp), kk = (int)(idx % Kp);
-    float v = 0.f;
-    if (kk < k * k * cin) {
-      const int ci = kk % cin, kx = (kk / cin) % k, ky = kk / (cin * k);
-      v = w[(((size_t)co * cin + ci) * k + ky) * k + kx];
-    }
-    st_op(wg, idx, v, bf);
-    if (wgT) st_op(wgT, (size_t)kk * cout + co, v, bf);
-  }
-}
-int launch_conv_w_prep(const float* w, int cout, int cin, int k, int Kp, void* wg, void* wgT,
-                       bool op_bf16, cudaStream_t s) {
-  ::ddppo::launch_k(conv_w_prep_kernel, grid_for((size_t)cout * Kp), 256, 0, s, w, cout, cin, k, Kp, wg, wgT,
-                                                                 op_bf16 ? 1 : 0);
-  DDPPO_CHECK_LAUNCH();
-  return DDPPO_OK;
-}
-__global__ void conv_w_flip_kernel(const float* __restrict__ w, int cout, int cin, int k, void* wr,
-                                   int bf) {
-  DDPPO_PDL_ENTRY();
-  const size_t total = (size_t)cin * k * k * cout;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (size_t)gridDim.x * blockDim.x) {
-    const int co = (int)(idx % cout);
-    const int tap = (int)((idx / cout) % (k * k));
-    const int ci = (int)(idx / ((size_t)cout * k * k));
-    const int ky = tap / k, kx = tap % k;
-    st_op(wr, idx, w[(((size_t)co * cin + ci) * k + (k - 1 - ky)) * k + (k - 1 - kx)], bf);
-  }
-}
-int launch_conv_w_flip(const float* w, int cout, int cin, int k, void* wr, bool op_bf16,
-                       cudaStream_t s) {
-  ::ddppo::launch_k(conv_w_flip_kernel, grid_for((size_t)cin * k * k * cout), 256, 0, s, w, cout, cin, k, wr,
-                                                                          op_bf16 ? 1 : 0);
-  DDPPO_CHECK_LAUNCH();
-  return DDPPO_OK;
-}
 __global__ void conv_w_grad_kernel(const float* __restrict__ dwg, int cout, int cin, int k, int Kp,
                                    float* __restrict__ dw) {
   DDPPO_PDL_ENTRY();
@@ -1036,26 +959,6 @@ __global__ void conv_w_grad_kernel(const float* __restrict__ dwg, int cout, int 
 int launch_conv_w_grad(const float* dwg, int cout, int cin, int k, int Kp, float* dw,
                        cudaStream_t s) {
   ::ddppo::launch_k(conv_w_grad_kernel, grid_for((size_t)cout * cin * k * k), 256, 0, s, dwg, cout, cin, k, Kp, dw);
-  DDPPO_CHECK_LAUNCH();
-  return DDPPO_OK;
-}
-__global__ void vis_w_prep_kernel(const float* __restrict__ w, int H, int C, int HW, void* wg,
-                                  void* wgT, int bf) {
-  DDPPO_PDL_ENTRY();
-  const int F = C * HW;
-  const size_t total = (size_t)H * F;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (size_t)gridDim.x * blockDim.x) {
-    const int h = (int)(idx / F), jg = (int)(idx % F);
-    const int c = jg % C, hw = jg / C;
-    const float v = w[(size_t)h * F + (size_t)c * HW + hw];
-    st_op(wg, idx, v, bf);
-    if (wgT) st_op(wgT, (size_t)jg * H + h, v, bf);
-  }
-}
-int launch_vis_w_prep(const float* w, int H, int C, int HW, void* wg, void* wgT, bool op_bf16,
-                      cudaStream_t s) {
-  ::ddppo::launch_k(vis_w_prep_kernel, grid_for((size_t)H * C * HW), 256, 0, s, w, H, C, HW, wg, wgT, op_bf16 ? 1 : 0);
   DDPPO_CHECK_LAUNCH();
   return DDPPO_OK;
 }
@@ -1076,18 +979,6 @@ int launch_vis_w_grad(const float* dwg, int H, int C, int HW, float* dw, cudaStr
   DDPPO_CHECK_LAUNCH();
   return DDPPO_OK;
 }
-__global__ void add_vec_kernel(const float* a, const float* b, float* out, int n) {
-  DDPPO_PDL_ENTRY();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = a[i] + b[i];
-}
-int launch_add_vec(const float* a, const float* b, float* out, int n, cudaStream_t s) {
-  if (!n) return DDPPO_OK;
-  ::ddppo::launch_k(add_vec_kernel, nblk(n, 256), 256, 0, s, a, b, out, n);
-  DDPPO_CHECK_LAUNCH();
-  return DDPPO_OK;
-}
-
 // ---------------------------------------------------------------- init
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
   z += 0x9E3779B97F4A7C15ull;

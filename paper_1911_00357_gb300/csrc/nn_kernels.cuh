@@ -20,9 +20,6 @@ int launch_im2col(const ConvGeom& g, const void* x, bool x_bf16, void* col, bool
                   bool transposed, cudaStream_t s);
 // col2im: dx[n, iy, ix, c] (+)= sum of dcol over the (ky, kx) that read it
 int launch_col2im(const ConvGeom& g, const float* dcol, float* dx, bool accumulate, cudaStream_t s);
-// out[c, r] = in[r, c]
-int launch_transpose(const void* in, bool in_bf16, void* out, bool out_bf16, int R, int Cc,
-                     int ld_in, cudaStream_t s);
 // fp32 -> op dtype copy (or plain copy)
 int launch_cast(const float* in, void* out, bool out_bf16, size_t n, cudaStream_t s);
 
@@ -255,20 +252,27 @@ int launch_vis_relu_bwd(int N, int H, const float* dx, int lddx, const void* x, 
 int launch_gather_rows(const void* in, void* out, const int32_t* idx, int T, int Ein, int Eout,
                        size_t bytes, cudaStream_t s);
 
-// weight preparation and gradient scatter between canonical and GEMM layouts
-int launch_conv_w_prep(const float* w, int cout, int cin, int k, int Kp, void* wg, void* wgT,
+// One weight tensor's operand copies (wprep.cu): source rows x (cin x kk) at params + src,
+// wg [rows][kk][cin] with leading dimension ld, wgT [kk][cin][rows] or null, wgR [cin][kk
+// reversed][rows] or null (the kernel of the input gradient of a stride-1 'same'
+// convolution, itself a convolution of the output gradient). kk = 0: the fp32 sum of the
+// vectors at src and src2 (rows elements) into wg. first: the first block of the entry.
+struct WPrep {
+  int64_t src = 0, src2 = 0;
+  int rows = 0, cin = 0, kk = 0, ld = 0, first = 0;
+  void* wg = nullptr;
+  void* wgT = nullptr;
+  void* wgR = nullptr;
+};
+int weight_prep_blocks(const WPrep& e);
+// every entry of table [dev]; entry [dev] maps a block to its entry
+int launch_weight_prep(const WPrep* table, const uint16_t* entry, int blocks, const float* params,
                        bool op_bf16, cudaStream_t s);
-// wr[ci, (ky*k + kx)*cout + co] = w[co, ci, k-1-ky, k-1-kx]: the kernel of the input
-// gradient of a stride-1 'same' convolution, itself a convolution of the output gradient
-int launch_conv_w_flip(const float* w, int cout, int cin, int k, void* wr, bool op_bf16,
-                       cudaStream_t s);
+// gradient scatter from the GEMM layouts to the canonical ones
 int launch_conv_w_grad(const float* dwg, int cout, int cin, int k, int Kp, float* dw,
                        cudaStream_t s);
 // vis FC: canonical column j = c*HW + hw  <->  GEMM column hw*C + c
-int launch_vis_w_prep(const float* w, int H, int C, int HW, void* wg, void* wgT, bool op_bf16,
-                      cudaStream_t s);
 int launch_vis_w_grad(const float* dwg, int H, int C, int HW, float* dw, cudaStream_t s);
-int launch_add_vec(const float* a, const float* b, float* out, int n, cudaStream_t s);
 
 // deterministic parameter init from the counter hash
 int launch_init_uniform(float* p, size_t n, float lo, float hi, uint64_t seed, uint64_t stream,
