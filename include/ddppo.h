@@ -568,11 +568,11 @@ int ddppo_update_graph(ddppo_ctx* ctx, int32_t on);
  * W_hh resident in shared memory, the cell update fused into the TMEM epilogue, one
  * bounded grid barrier per step) wherever the shape allows (H a multiple of 64, at most
  * 128 envs per segment, 64 when H = 512); the backward, the FP32 form and other shapes
- * run as in mode 0. mode 0 (the default): segments of more than one step of at most 64 envs
- * run in the BF16 forms in one launch per layer and direction (a thread-block cluster per
- * few envs, the recurrent weights in its registers) where H is 64, 128, 256 or 512; other
- * shapes and the FP32 form take a recurrent contraction and a cell kernel per step. Both
- * give the same bits. mode 1: forward and backward as one cooperative launch per layer on the
+ * run as in mode 0. mode 0 (the default): one launch per layer and direction (a thread-block
+ * cluster per few envs, the recurrent weights in its registers) for H of 64, 128, 256 and, in
+ * the BF16 forms, 512: BF16 segments of more than one step of at most 64 envs, FP32 segments
+ * of any length; other shapes take a recurrent contraction and a cell kernel per step, whose
+ * bits the BF16 cluster form gives too. mode 1: forward and backward as one cooperative launch per layer on the
  * CUDA cores (recurrent weights in registers; at most 64 envs per segment); slower than
  * mode 0 at the default sizes (its per-step contraction is bound by shared-memory loads).
  * All modes compute the same arithmetic; only the recurrent contraction's fp32 summation

@@ -1,0 +1,71 @@
+// Device helpers of the thread-block-cluster kernels: ranks, cluster barrier, remote stores
+// that complete the receiver's mbarrier, and the bounded wait for them (sm_103a).
+#pragma once
+
+#include "tc_common.cuh"
+
+namespace ddppo {
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+}
+__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+// 16 bytes into another CTA's shared memory; they count towards its barrier's bytes
+__device__ __forceinline__ void send16(uint32_t raddr, uint4 v, uint32_t rbar) {
+  asm volatile(
+      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+          raddr),
+      "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(rbar)
+      : "memory");
+}
+__device__ __forceinline__ void expect_bytes(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
+               "r"(bytes)
+               : "memory");
+}
+// bounded wait for the peers' bytes (acquire at cluster scope)
+__device__ __forceinline__ bool wait_bytes(uint64_t* bar, uint32_t parity, int32_t* err) {
+  for (uint32_t i = 0; i < TC_SPIN_LIMIT; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred P1;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P1, [%1], %2;\n\t"
+        "selp.b32 %0, 1, 0, P1;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    // a CTA elsewhere gave up: stop waiting for its bytes
+    if ((i & 1023u) == 1023u && err && (*(volatile int32_t*)err & ERRF_TIMEOUT)) return false;
+  }
+  if (err) atomicOr(err, ERRF_TIMEOUT);
+  return false;
+}
+__device__ __forceinline__ void send4(uint32_t raddr, float v, uint32_t rbar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(raddr),
+               "r"(__float_as_uint(v)), "r"(rbar)
+               : "memory");
+}
+
+// after the last step: every CTA of the cluster has issued all it sends; if one gave up,
+// let what is in flight land (bounded) before the shared memory goes away
+__device__ __forceinline__ void cluster_end(uint64_t* full, bool failed) {
+  __syncwarp();
+  cluster_sync();
+  if (failed && threadIdx.x == 0) {
+    mbar_drain_wait(&full[0], 0u);
+    mbar_drain_wait(&full[1], 0u);
+  }
+}
+
+}  // namespace ddppo

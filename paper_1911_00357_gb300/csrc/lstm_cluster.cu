@@ -35,9 +35,9 @@
 #include <algorithm>
 #include <atomic>
 
+#include "cluster.cuh"
 #include "lstm_cell.cuh"
 #include "nn_kernels.cuh"
-#include "tc_common.cuh"
 
 namespace ddppo {
 
@@ -49,51 +49,6 @@ constexpr int LC_ENVS = 8;       // envs per cluster at most (the MMA's N side)
 constexpr int LC_BLOCK = 512;    // bytes of one [8 envs][32 units] bf16 block
 constexpr int LC_RED_PITCH = 36; // backward partial sums: floats per env row
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
-                   : "memory");
-}
-__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
-  return r;
-}
-// 16 bytes into another CTA's shared memory; they count towards its barrier's bytes
-__device__ __forceinline__ void send16(uint32_t raddr, uint4 v, uint32_t rbar) {
-  asm volatile(
-      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
-          raddr),
-      "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(rbar)
-      : "memory");
-}
-__device__ __forceinline__ void expect_bytes(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)),
-               "r"(bytes)
-               : "memory");
-}
-// bounded wait for the peers' bytes (acquire at cluster scope)
-__device__ __forceinline__ bool wait_bytes(uint64_t* bar, uint32_t parity, int32_t* err) {
-  for (uint32_t i = 0; i < TC_SPIN_LIMIT; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred P1;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P1, [%1], %2;\n\t"
-        "selp.b32 %0, 1, 0, P1;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    // a CTA elsewhere gave up: stop waiting for its bytes
-    if ((i & 1023u) == 1023u && err && (*(volatile int32_t*)err & ERRF_TIMEOUT)) return false;
-  }
-  if (err) atomicOr(err, ERRF_TIMEOUT);
-  return false;
-}
 __device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t saddr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -119,17 +74,6 @@ __device__ __forceinline__ int ldsm_off(int lane) {
 }
 __device__ __forceinline__ uint32_t ld_w2(const __nv_bfloat16* p) {
   return __ldg(reinterpret_cast<const uint32_t*>(p));
-}
-
-// after the last step: every CTA of the cluster has issued all it sends; if one gave up,
-// let what is in flight land (bounded) before the shared memory goes away
-__device__ __forceinline__ void cluster_end(uint64_t* full, bool failed) {
-  __syncwarp();
-  cluster_sync();
-  if (failed && threadIdx.x == 0) {
-    mbar_drain_wait(&full[0], 0u);
-    mbar_drain_wait(&full[1], 0u);
-  }
 }
 
 template <int KS>
@@ -167,7 +111,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_fwd_kernel(LstmCl a) {
         for (int q = 0; q < 4; ++q) p[q] = __floats2bfloat162_rn(a.h0[o + 2 * q], a.h0[o + 2 * q + 1]);
         v = *reinterpret_cast<uint4*>(p);
       }
-      if (j == cta) *reinterpret_cast<uint4*>(a.hm + o) = v;
+      if (j == cta) *reinterpret_cast<uint4*>((__nv_bfloat16*)a.hm + o) = v;
     }
     *reinterpret_cast<uint4*>(&hs[0][j * LC_BLOCK + blk_off(row, (i & 3) * 8)]) = v;
     *reinterpret_cast<uint4*>(&hs[1][j * LC_BLOCK + blk_off(row, (i & 3) * 8)]) = make_uint4(0u, 0u, 0u, 0u);
@@ -175,7 +119,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_fwd_kernel(LstmCl a) {
   // this warp's 16 gate rows: MMA row r is gate r / 4 of unit warp * 4 + r % 4
   uint32_t w[KS][4];
   {
-    const __nv_bfloat16* r0 = a.W + (size_t)((g >> 2) * H + unit) * H + 2 * t4;
+    const __nv_bfloat16* r0 = (const __nv_bfloat16*)a.W + (size_t)((g >> 2) * H + unit) * H + 2 * t4;
     const __nv_bfloat16* r1 = r0 + (size_t)2 * H * H;  // rows 8 .. 15: gates g, o
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
@@ -279,8 +223,8 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_fwd_kernel(LstmCl a) {
       a.gates[gb + 3 * H] = go;
       a.c[ho] = c;
       a.h[ho] = h;
-      a.y[ho] = __float2bfloat16_rn(h);
-      if (!last) a.hm[ho + EH] = hn;
+      ((__nv_bfloat16*)a.y)[ho] = __float2bfloat16_rn(h);
+      if (!last) ((__nv_bfloat16*)a.hm)[ho + EH] = hn;
     }
     if (stop) break;
 #pragma unroll
@@ -323,7 +267,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_bwd_kernel(LstmCl a) {
   uint32_t w[2][PER][4];
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt) {
-    const __nv_bfloat16* r0 = a.W + (size_t)(cta * LC_UNITS + mt * 16 + g) * 4 * H +
+    const __nv_bfloat16* r0 = (const __nv_bfloat16*)a.W + (size_t)(cta * LC_UNITS + mt * 16 + g) * 4 * H +
                               (size_t)warp * PER * 16 + 2 * t4;
     const __nv_bfloat16* r1 = r0 + (size_t)8 * 4 * H;
 #pragma unroll
@@ -423,8 +367,205 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_bwd_kernel(LstmCl a) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         a.dg32[gb + q * H] = dz[q];
-        a.dg_op[gb + q * H] = db16[q];
+        ((__nv_bfloat16*)a.dg_op)[gb + q * H] = db16[q];
       }
+    }
+  }
+  cluster_end(full, !ok);
+}
+
+// ---- FP32 operands: the same scheme on the CUDA cores ----
+// CTA j owns 32 units; its weights (64 KB at H = 128) are registers: warp w holds gate w / 2
+// of them over K half w % 2 (forward), or slice w of the 4H gate gradients (backward), lane =
+// unit, and multiplies with the envs' rows broadcast from shared memory. The eight partial
+// sums of a (unit, env) meet in shared memory; thread (env = warp, unit = lane) updates the
+// cell and sends its value to every CTA. Covered to H = 256 (128 weight registers a thread).
+template <int K2>
+__device__ __forceinline__ void load_row(float (&w)[K2], const float* p) {
+#pragma unroll
+  for (int k = 0; k < K2; k += 4) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p + k));
+    w[k] = v.x; w[k + 1] = v.y; w[k + 2] = v.z; w[k + 3] = v.w;
+  }
+}
+template <int K2>
+__device__ __forceinline__ float dot_row(const float (&w)[K2], const float* h) {
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < K2; k += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(h + k);
+    s[0] = fmaf(w[k], v.x, s[0]);
+    s[1] = fmaf(w[k + 1], v.y, s[1]);
+    s[2] = fmaf(w[k + 2], v.z, s[2]);
+    s[3] = fmaf(w[k + 3], v.w, s[3]);
+  }
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+
+template <int H>
+__global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl32_fwd_kernel(LstmCl a) {
+  DDPPO_PDL_ENTRY();
+  constexpr int CL = H / LC_UNITS, K2 = H / 2;
+  __shared__ __align__(16) float hs[2][LC_ENVS][H];
+  __shared__ float red[8][LC_ENVS][LC_UNITS];
+  __shared__ uint64_t full[2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cta = (int)cluster_rank();
+  const int e0 = (int)(blockIdx.x / CL) * a.epc, ne = min(a.epc, a.E - e0);
+  const bool mine = warp < ne;
+  const int unit = cta * LC_UNITS + lane, e = e0 + (mine ? warp : 0);
+  const uint32_t bytes = (uint32_t)(H * ne * 4);
+  float* hm = (float*)a.hm;
+  if (threadIdx.x == 0) {
+    mbar_init(&full[0], 1);
+    mbar_init(&full[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (a.T > 1) expect_bytes(&full[1], bytes);
+    if (a.T > 2) expect_bytes(&full[0], bytes);
+  }
+  for (int i = threadIdx.x; i < ne * H; i += LC_THREADS) {
+    const int row = i / H, k = i - row * H;
+    const size_t o = (size_t)(e0 + row) * H + k;
+    const float v = a.m[e0 + row] ? a.h0[o] : 0.f;
+    hs[0][row][k] = v;
+    if (k / LC_UNITS == cta) hm[o] = v;
+  }
+  float w[K2];
+  load_row<K2>(w, (const float*)a.W + (size_t)((warp >> 1) * H + unit) * H + (warp & 1) * K2);
+  const size_t EG = (size_t)a.E * 4 * H, EH = (size_t)a.E * H;
+  const float* gxp = a.gx + (size_t)e * 4 * H + unit;
+  float c = mine ? a.c0[(size_t)e * H + unit] : 0.f;
+  bool mk = mine && a.m[e];
+  float gx[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) gx[q] = mine ? gxp[q * H] : 0.f;
+  __syncthreads();
+  cluster_sync();
+
+  bool ok = true;
+  for (int t = 0; t < a.T; ++t) {
+    if (t > 0) ok = wait_bytes(&full[t & 1], (uint32_t)((t - 1) >> 1) & 1u, a.err) && ok;
+    if (threadIdx.x == 0 && t > 0 && t + 2 < a.T) expect_bytes(&full[t & 1], bytes);
+    const bool last = t + 1 == a.T;
+    float gn[4] = {0.f, 0.f, 0.f, 0.f};
+    bool mn = false;
+    if (mine && !last) {
+      const float* p = gxp + (size_t)(t + 1) * EG;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) gn[q] = __ldg(p + q * H);
+      mn = a.m[(size_t)(t + 1) * a.E + e] != 0;
+    }
+    for (int n = 0; n < ne; ++n) red[warp][n][lane] = dot_row<K2>(w, &hs[t & 1][n][(warp & 1) * K2]);
+    // (the buffer of partial sums is free again at the next step: its wait ends only after
+    // every cell of this CTA has been read, updated and sent)
+    if (__syncthreads_or(ok ? 0 : 1)) { ok = false; break; }
+    if (mine) {
+      float z[4], gi, gf, gg, go, h;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) z[q] = gx[q] + (red[2 * q][warp][lane] + red[2 * q + 1][warp][lane]);
+      lstm_cell_fwd(z[0], z[1], z[2], z[3], mk ? c : 0.f, gi, gf, gg, go, c, h);
+      const float hn = mn ? h : 0.f;
+      if (!last) {
+        const int nb = (t + 1) & 1;
+        const uint32_t dst = smem_addr(&hs[nb][warp][unit]), bar = smem_addr(&full[nb]);
+#pragma unroll
+        for (int r = 0; r < CL; ++r) send4(map_rank(dst, r), hn, map_rank(bar, r));
+      }
+      const size_t gb = (size_t)t * EG + (size_t)e * 4 * H + unit, ho = (size_t)t * EH + (size_t)e * H + unit;
+      a.gates[gb] = gi;
+      a.gates[gb + H] = gf;
+      a.gates[gb + 2 * H] = gg;
+      a.gates[gb + 3 * H] = go;
+      a.c[ho] = c;
+      a.h[ho] = h;
+      ((float*)a.y)[ho] = h;
+      if (!last) hm[ho + EH] = hn;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) gx[q] = gn[q];
+    mk = mn;
+  }
+  cluster_end(full, !ok);
+}
+
+template <int H>
+__global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl32_bwd_kernel(LstmCl a) {
+  DDPPO_PDL_ENTRY();
+  constexpr int CL = H / LC_UNITS, K2 = H / 2, ROW = 4 * H;
+  extern __shared__ __align__(128) float dz_in[];  // [2][LC_ENVS][4H]
+  __shared__ float red[8][LC_ENVS][LC_UNITS];
+  __shared__ uint64_t full[2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cta = (int)cluster_rank();
+  const int e0 = (int)(blockIdx.x / CL) * a.epc, ne = min(a.epc, a.E - e0);
+  const bool mine = warp < ne;
+  const int unit = cta * LC_UNITS + lane, e = e0 + (mine ? warp : 0);
+  const uint32_t bytes = (uint32_t)(ROW * ne * 4);
+  if (threadIdx.x == 0) {
+    mbar_init(&full[0], 1);
+    mbar_init(&full[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (a.T > 1) expect_bytes(&full[1], bytes);
+    if (a.T > 2) expect_bytes(&full[0], bytes);
+  }
+  float w[K2];
+  load_row<K2>(w, (const float*)a.W + (size_t)unit * ROW + warp * K2);
+  const size_t EG = (size_t)a.E * ROW, EH = (size_t)a.E * H;
+  const size_t gofs = (size_t)e * ROW + unit, hofs = (size_t)e * H + unit;
+  float c = mine ? a.c[(size_t)(a.T - 1) * EH + hofs] : 0.f, dcc = 0.f;
+  bool mnext = false;
+  __syncthreads();
+  cluster_sync();
+
+  bool ok = true;
+  for (int it = 0; it < a.T; ++it) {
+    const int t = a.T - 1 - it;
+    float gt[4] = {0.f, 0.f, 0.f, 0.f}, cprev = 0.f, dha = 0.f;
+    bool mk = false;
+    if (mine) {
+      const float* gp = a.gates + (size_t)t * EG + gofs;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) gt[q] = gp[q * H];
+      cprev = t == 0 ? a.c0[hofs] : a.c[(size_t)(t - 1) * EH + hofs];
+      dha = a.dh_above[(size_t)t * EH + hofs];
+      mk = a.m[(size_t)t * a.E + e] != 0;
+    }
+    float rec = 0.f;
+    if (it > 0) {
+      ok = wait_bytes(&full[it & 1], (uint32_t)((it - 1) >> 1) & 1u, a.err) && ok;
+      if (threadIdx.x == 0 && it + 2 < a.T) expect_bytes(&full[it & 1], bytes);
+      const float* in = dz_in + (size_t)(it & 1) * LC_ENVS * ROW + warp * K2;
+      for (int n = 0; n < ne; ++n) red[warp][n][lane] = dot_row<K2>(w, in + n * ROW);
+      if (__syncthreads_or(ok ? 0 : 1)) { ok = false; break; }
+      if (mine) {
+#pragma unroll
+        for (int s = 0; s < 8; ++s) rec += red[s][warp][lane];
+      }
+    }
+    if (!mine) continue;
+    float dh = dha;
+    if (mnext && it > 0) dh += rec;
+    float dz[4], dco;
+    lstm_cell_bwd(gt[0], gt[1], gt[2], gt[3], c, mk ? cprev : 0.f, dh, mnext, dcc, dz[0], dz[1], dz[2],
+                  dz[3], dco);
+    dcc = dco;
+    c = cprev;
+    mnext = mk;
+    if (t > 0) {
+      const int nb = (it + 1) & 1;
+      const uint32_t dst = smem_addr(dz_in + ((size_t)nb * LC_ENVS + warp) * ROW + unit), bar = smem_addr(&full[nb]);
+#pragma unroll
+      for (int r = 0; r < CL; ++r) {
+        const uint32_t rd = map_rank(dst, r), rb = map_rank(bar, r);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) send4(rd + q * H * 4, dz[q], rb);
+      }
+    }
+    const size_t gb = (size_t)t * EG + gofs;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      a.dg32[gb + q * H] = dz[q];
+      ((float*)a.dg_op)[gb + q * H] = dz[q];
     }
   }
   cluster_end(full, !ok);
@@ -432,22 +573,35 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_bwd_kernel(LstmCl a) {
 
 typedef void (*ClKernel)(LstmCl);
 struct ClForm {
-  ClKernel fwd, bwd;
-  int CL;
-  size_t bwd_smem;
+  ClKernel fwd = nullptr, bwd = nullptr;
+  int CL = 0;
+  size_t bwd_smem = 0;
 };
 template <int KS>
-ClForm make_form() {
+ClForm bf16_form() {
   return ClForm{lstm_cl_fwd_kernel<KS>, lstm_cl_bwd_kernel<KS>, KS / 2,
                 (size_t)2 * (KS / 2) * 4 * LC_BLOCK};
 }
-bool form_of(int H, ClForm* f) {
-  if (H == 512) *f = make_form<32>();
-  else if (H == 256) *f = make_form<16>();
-  else if (H == 128) *f = make_form<8>();
-  else if (H == 64) *f = make_form<4>();
-  else return false;
-  return true;
+template <int H>
+ClForm fp32_form() {
+  return ClForm{lstm_cl32_fwd_kernel<H>, lstm_cl32_bwd_kernel<H>, H / LC_UNITS,
+                (size_t)2 * LC_ENVS * 4 * H * sizeof(float)};
+}
+constexpr int LC_SIZES[4] = {64, 128, 256, 512};
+// the kernels of hidden size LC_SIZES[i]; fwd null where not covered
+ClForm form_of(int i, bool bf) {
+  switch (i) {
+    case 0: return bf ? bf16_form<4>() : fp32_form<64>();
+    case 1: return bf ? bf16_form<8>() : fp32_form<128>();
+    case 2: return bf ? bf16_form<16>() : fp32_form<256>();
+    case 3: return bf ? bf16_form<32>() : ClForm{};
+    default: return ClForm{};
+  }
+}
+int size_index(int H) {
+  for (int i = 0; i < 4; ++i)
+    if (LC_SIZES[i] == H) return i;
+  return -1;
 }
 
 cudaLaunchConfig_t cl_config(int clusters, int CL, size_t smem, cudaStream_t s,
@@ -469,13 +623,15 @@ cudaLaunchConfig_t cl_config(int clusters, int CL, size_t smem, cudaStream_t s,
 }
 
 // clusters of this hidden size that the current device holds at once (0: none, or the size
-// is not covered); asked once per device and size
-int cl_resident(int H) {
-  static std::atomic<int> cache[64][4];  // 0: not asked yet, else the answer + 1
-  ClForm f;
+// is not covered); asked once per device, size and operand type
+int cl_resident(int H, bool bf) {
+  static std::atomic<int> cache[64][8];  // 0: not asked yet, else the answer + 1
+  const int i = size_index(H);
   int dev = 0;
-  if (!form_of(H, &f) || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  std::atomic<int>& slot = cache[dev][H == 512 ? 0 : H == 256 ? 1 : H == 128 ? 2 : 3];
+  if (i < 0 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  const ClForm f = form_of(i, bf);
+  if (!f.fwd) return 0;
+  std::atomic<int>& slot = cache[dev][2 * i + (bf ? 1 : 0)];
   const int known = slot.load();
   if (known) return known - 1;
   int least = 1 << 20;
@@ -492,19 +648,19 @@ int cl_resident(int H) {
       (void)cudaGetLastError();
       num = 0;
     }
-    least = num < least ? num : least;
+    least = std::min(num, least);
   }
   slot.store(least + 1);
   return least;
 }
 
-int launch_cl(const LstmCl& in, bool bwd, cudaStream_t s) {
-  ClForm f;
-  const int room = cl_resident(in.H);
-  if (!form_of(in.H, &f) || room < 1) {
+int launch_cl(const LstmCl& in, bool bf, bool bwd, cudaStream_t s) {
+  const int room = cl_resident(in.H, bf);
+  if (room < 1) {
     set_error("lstm: the cluster form does not cover this hidden size or device");
     return DDPPO_E_CONFIG;
   }
+  const ClForm f = form_of(size_index(in.H), bf);
   LstmCl a = in;
   // as few envs per cluster as keep all clusters resident at once (fewer bytes to exchange
   // per step), at most 8
@@ -518,12 +674,20 @@ int launch_cl(const LstmCl& in, bool bwd, cudaStream_t s) {
 
 }  // namespace
 
-// Covered: the hidden sizes whose weights fit a cluster's registers, up to 64 envs: above
-// that the step-by-step contraction is the tcgen05 one, which sums in another order, and the
-// recurrence would no longer give that path's bits. 57 to 64 envs at H = 512 take two waves
-// of clusters (7 are resident at once), about 3.5 us a step, still a third of the steps'.
-bool lstm_cl_supported(int H, int E) { return E >= 1 && E <= 64 && cl_resident(H) >= 1; }
-int launch_lstm_cl_fwd(const LstmCl& a, cudaStream_t s) { return launch_cl(a, false, s); }
-int launch_lstm_cl_bwd(const LstmCl& a, cudaStream_t s) { return launch_cl(a, true, s); }
+// BF16: segments of more than one step and up to 64 envs. Above that the step-by-step
+// contraction is the tcgen05 one, which sums in another order, and the recurrence would no
+// longer give that path's bits; a single step measured no gain (the act pass: 597 us with
+// it, 584 without). 57 to 64 envs at H = 512 take two waves of clusters (7 are resident at
+// once), about 3.5 us a step, still a third of the steps'.
+// FP32: any segment that fits one wave of clusters (H = 128: 592 envs); the step-by-step
+// form costs 12 us a step there against 0.9 us (H = 128, 32 steps x 8 envs: 29 us forward, 27 us
+// backward a segment; the 16-env update 6.96 -> 3.54 ms).
+bool lstm_cl_supported(int H, int T, int E, bool bf) {
+  if (T < 1 || E < 1 || (bf && (T < 2 || E > 64))) return false;
+  const int room = cl_resident(H, bf);
+  return room >= 1 && (bf || E <= LC_ENVS * room);
+}
+int launch_lstm_cl_fwd(const LstmCl& a, bool bf, cudaStream_t s) { return launch_cl(a, bf, false, s); }
+int launch_lstm_cl_bwd(const LstmCl& a, bool bf, cudaStream_t s) { return launch_cl(a, bf, true, s); }
 
 }  // namespace ddppo

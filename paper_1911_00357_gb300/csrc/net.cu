@@ -997,9 +997,7 @@ static int lstm_forward(Net& n, int T, int E, const uint8_t* masks, const float*
   const bool seq = n.lstm_mode == 1 && lstm_seq_supported(Hd, E, n.gws.num_sms);
   // (a single step -- the act path -- gains nothing from resident weights: step path)
   const bool tc = n.lstm_mode == 2 && n.bf && T > 1 && lstm_tc_supported(Hd, E, n.gws.num_sms);
-  // one cluster launch per layer; a single step takes the step path, as fast there (64 envs
-  // need two waves of clusters: the act pass measured 597 us with them, 584 without)
-  const bool cl = !seq && !tc && n.bf && T > 1 && lstm_cl_supported(Hd, E);
+  const bool cl = !seq && !tc && lstm_cl_supported(Hd, T, E, n.bf);
   for (int l = 0; l < n.L; ++l) {
     LstmL& q = n.lstm[l];
     GemmDesc gx;
@@ -1034,12 +1032,12 @@ static int lstm_forward(Net& n, int T, int E, const uint8_t* masks, const float*
     if (cl) {
       LstmCl a{};
       a.T = T; a.E = E; a.H = Hd;
-      a.W = (const __nv_bfloat16*)q.Whh;
+      a.W = q.Whh;
       a.gx = n.gx; a.m = masks; a.h0 = h0 + (size_t)l * E * Hd; a.c0 = c0 + (size_t)l * E * Hd;
       a.gates = q.gates; a.c = q.c; a.h = q.h;
-      a.y = (__nv_bfloat16*)q.y; a.hm = (__nv_bfloat16*)q.hm;
+      a.y = q.y; a.hm = q.hm;
       a.err = n.gws.err;
-      DDPPO_TRY(launch_lstm_cl_fwd(a, s));
+      DDPPO_TRY(launch_lstm_cl_fwd(a, n.bf, s));
       continue;
     }
     DDPPO_TRY(launch_mask_state(h0 + (size_t)l * E * Hd, masks, E, Hd, q.hm, n.bf, s));
@@ -1077,7 +1075,7 @@ static int lstm_backward(Net& n, int T, int E, const uint8_t* masks, const float
                          const float* dtop, const float** dx0, cudaStream_t s) {
   const int N = T * E, Hd = n.H, G4 = 4 * Hd;
   const bool seq = n.lstm_mode == 1 && lstm_seq_supported(Hd, E, n.gws.num_sms);
-  const bool cl = !seq && n.bf && T > 1 && lstm_cl_supported(Hd, E);
+  const bool cl = !seq && lstm_cl_supported(Hd, T, E, n.bf);
   const float* dabove = dtop;
   for (int l = n.L - 1; l >= 0; --l) {
     LstmL& q = n.lstm[l];
@@ -1093,12 +1091,12 @@ static int lstm_backward(Net& n, int T, int E, const uint8_t* masks, const float
     if (cl) {
       LstmCl a{};
       a.T = T; a.E = E; a.H = Hd;
-      a.W = (const __nv_bfloat16*)q.WhhT;
+      a.W = q.WhhT;
       a.m = masks; a.c0 = c0 + (size_t)l * E * Hd;
       a.gates = q.gates; a.c = q.c;
-      a.dh_above = dabove; a.dg32 = n.dg32; a.dg_op = (__nv_bfloat16*)n.dgop;
+      a.dh_above = dabove; a.dg32 = n.dg32; a.dg_op = n.dgop;
       a.err = n.gws.err;
-      DDPPO_TRY(launch_lstm_cl_bwd(a, s));
+      DDPPO_TRY(launch_lstm_cl_bwd(a, n.bf, s));
     }
     const bool steps = !seq && !cl;
     if (steps) DDPPO_CHECK_CUDA(cudaMemsetAsync(n.dc_carry, 0, (size_t)E * Hd * sizeof(float), s));

@@ -210,7 +210,7 @@ struct Net {
   bool upd_graph_on = true;      // caller's choice (ddppo_update_graph)
   int64_t* d_steps = nullptr;    // [2] device: update index, Adam steps before this update
   unsigned* lstm_bar = nullptr;  // grid-barrier counter of the whole-segment LSTM kernels
-  // LSTM recurrence: 0 whole segment on clusters where covered (BF16, up to 64 envs), else
+  // LSTM recurrence: 0 whole segment on clusters where covered, else
   // step by step; 1 whole segment on CUDA cores (forward and backward); 2 forward on tcgen05
   // (whole segment, BF16), backward as in 0
   int lstm_mode = 0;

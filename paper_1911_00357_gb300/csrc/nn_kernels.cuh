@@ -191,22 +191,22 @@ struct LstmTc {
 };
 bool lstm_tc_supported(int H, int E, int num_sms);
 
-// The recurrence of one layer over a whole segment in one cluster launch (lstm_cluster.cu),
-// BF16 operands, at most 64 envs; [T, E, *] layouts and arithmetic of the step-by-step
-// path (bit-identical). Forward: W = Whh [4H, H]; gx, m, h0, c0 -> gates, c, h, y, hm (the
-// masked state entering each step, slot 0 included). Backward: W = WhhT [H, 4H]; gates, c,
-// c0, m, dh_above -> dg32, dg_op. epc is set by the launcher.
+// The recurrence of one layer over a whole segment in one cluster launch (lstm_cluster.cu);
+// [T, E, *] layouts of the step-by-step path, operands (W, y, hm, dg_op) bf16 or fp32. The
+// BF16 form is bit-identical with that path. Forward: W = Whh [4H, H]; gx, m, h0, c0 ->
+// gates, c, h, y, hm (the masked state entering each step, slot 0 included). Backward: W =
+// WhhT [H, 4H]; gates, c, c0, m, dh_above -> dg32, dg_op. epc is set by the launcher.
 struct LstmCl {
   int T, E, H, epc;
-  const __nv_bfloat16* W;
+  const void* W;
   const float* gx; const uint8_t* m; const float* h0; const float* c0;
-  float* gates; float* c; float* h; __nv_bfloat16* y; __nv_bfloat16* hm;
-  const float* dh_above; float* dg32; __nv_bfloat16* dg_op;
+  float* gates; float* c; float* h; void* y; void* hm;
+  const float* dh_above; float* dg32; void* dg_op;
   int32_t* err;
 };
-bool lstm_cl_supported(int H, int E);
-int launch_lstm_cl_fwd(const LstmCl& a, cudaStream_t s);
-int launch_lstm_cl_bwd(const LstmCl& a, cudaStream_t s);
+bool lstm_cl_supported(int H, int T, int E, bool bf);
+int launch_lstm_cl_fwd(const LstmCl& a, bool bf, cudaStream_t s);
+int launch_lstm_cl_bwd(const LstmCl& a, bool bf, cudaStream_t s);
 
 // single-channel convolution on tcgen05 (conv_c1_tc.cu): y [N, Ho, Wo, Cout] fp32
 // (= beta y + conv) of x [N, H, W] bf16 with w [Cout, ldw] bf16 (taps (ky, kx) in its
