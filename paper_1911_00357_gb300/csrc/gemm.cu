@@ -240,6 +240,12 @@ int gemm(const GemmDesc& d, bool op_bf16, const GemmWorkspace& ws, cudaStream_t 
     rc = gemm_small(d, s);  // latency-bound small-M shapes: no tensor-memory pipeline
   } else if (op_bf16 && d.convw && conv_wgrad_halo_ok(*d.convw, d.B, d.A)) {
     rc = conv_wgrad_halo(*d.convw, d.B, d.A, (float*)d.C, d.ldc, d.beta, ws, s);
+  } else if (op_bf16 && d.convw && conv_wgrad_rows_ok(*d.convw, d.B, d.A, ws)) {
+    rc = conv_wgrad_rows(*d.convw, d.B, d.A, (float*)d.C, d.ldc, d.beta, ws, s);
+    if (ws.tc && ws.tc->on) {
+      ws.tc->launches += 1;
+      ws.tc->flops += 2.0 * d.M * d.N * d.K;
+    }
   } else if (op_bf16 && (d.conv || d.convw || gemm_tc_supported(d))) {
     rc = gemm_tc(d, ws, s);
     if (ws.tc && ws.tc->on) {

@@ -106,6 +106,11 @@ bool gemm_conv_supported(const ConvShape& c, const void* input);
 bool conv_wgrad_halo_ok(const ConvShape& c, const void* x, const void* dz);
 int conv_wgrad_halo(const ConvShape& c, const void* x, const void* dz, float* dw, int ldw, float beta,
                     const GemmWorkspace& ws, cudaStream_t s);
+// weight gradient of a 3x3 / stride-1 / pad-1 convolution, 64 -> 64 channels or multiples of
+// 128, every tap a shifted view of one staged box (wgrad_rows.cu); same result layout
+bool conv_wgrad_rows_ok(const ConvShape& c, const void* x, const void* dz, const GemmWorkspace& ws);
+int conv_wgrad_rows(const ConvShape& c, const void* x, const void* dz, float* dw, int ldw, float beta,
+                    const GemmWorkspace& ws, cudaStream_t s);
 // small-M BF16 contraction (gemm_small.cu): M <= 64, both operands K-major, K % 16 == 0
 bool gemm_small_supported(const GemmDesc& d);
 int gemm_small(const GemmDesc& d, cudaStream_t s);
