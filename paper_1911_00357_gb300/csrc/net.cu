@@ -279,8 +279,8 @@ static int alloc_encoder(Net& n) {
       const int HWi = X.c1.H * X.c1.W;
       DDPPO_TRY(conv_bufs(X.c1));
       DDPPO_TRY(conv_bufs(X.c3));
-      DDPPO_TRY(gn_bufs(X.n1, HWi, true));
-      DDPPO_TRY(gn_bufs(X.n2, X.HW, true));
+      DDPPO_TRY(gn_bufs(X.n1, HWi, !n.bf));  // BF16 form: only the bf16 copies are read
+      DDPPO_TRY(gn_bufs(X.n2, X.HW, !n.bf));
       DDPPO_TRY(gn_bufs(X.n3, X.HW, false));
       if (X.down) {
         DDPPO_TRY(conv_bufs(X.d));
@@ -317,13 +317,16 @@ static int alloc_encoder(Net& n) {
       if (n.kind != 1) break;
       DDPPO_TRY(conv_bufs(B.c1));
       DDPPO_TRY(conv_bufs(B.c2));
-      DDPPO_TRY(gn_bufs(B.n1, B.c1.Ho * B.c1.Wo, true));
+      // (in the BF16 form only the bf16 copy of this activation is read: the convolution's
+      // operand; the backward recomputes the ReLU's mask from the convolution output)
+      DDPPO_TRY(gn_bufs(B.n1, B.c1.Ho * B.c1.Wo, !n.bf));
       DDPPO_TRY(gn_bufs(B.n2, B.c2.Ho * B.c2.Wo, false));
       if (B.down) {
         DDPPO_TRY(conv_bufs(B.d));
         DDPPO_TRY(gn_bufs(B.nd, B.d.Ho * B.d.Wo, false));
       }
       DDPPO_TRY(nalloc(n, &B.y, NC * B.c2.Ho * B.c2.Wo * B.c2.cout));
+      if (B.c2.cout % 4 == 0) DDPPO_TRY(nalloc(n, &B.pos, NC * B.c2.Ho * B.c2.Wo * B.c2.cout / 4));
       if (n.bf) {
         DDPPO_TRY(nalloc(n, &B.y_bf, NC * B.c2.Ho * B.c2.Wo * B.c2.cout));
         DDPPO_TRY(nalloc(n, &B.n1.out_bf, NC * B.c1.Ho * B.c1.Wo * B.c1.cout));
@@ -654,7 +657,8 @@ static int conv_fwd(Net& n, ConvL& c, const void* in, bool in_bf16, int N, float
     return G(n, d, s);
   }
   const ConvGeom g = geom(c, N);
-  DDPPO_TRY(launch_im2col(g, in, in_bf16, n.col, n.bf, false, s));
+  if (n.bf && in_bf) DDPPO_TRY(launch_im2col(g, in_bf, true, n.col, n.bf, false, s));
+  else DDPPO_TRY(launch_im2col(g, in, in_bf16, n.col, n.bf, false, s));
   d.A = n.col; d.lda = c.Kp;
   return G(n, d, s);
 }
@@ -716,7 +720,8 @@ static int conv_bwd(Net& n, ConvL& c, const void* in, bool in_bf16, int N, const
 
 static int gn_fwd(Net& n, GNL& g, const float* z, int N, int HW, float* out, bool relu,
                   const float* resid, const GNL* gd, const float* zd, cudaStream_t s,
-                  __nv_bfloat16* out_bf = nullptr, uint8_t* out_f8 = nullptr, int f8_slot = -1) {
+                  __nv_bfloat16* out_bf = nullptr, uint8_t* out_f8 = nullptr, int f8_slot = -1,
+                  uint8_t* pos = nullptr) {
   const float eps = 1e-5f;
   GNApply a{};
   a.z = z; a.mean = g.mean; a.rstd = g.rstd;
@@ -728,6 +733,7 @@ static int gn_fwd(Net& n, GNL& g, const float* z, int N, int HW, float* out, boo
   }
   a.out = out;
   a.out_bf = out_bf;
+  a.pos = pos;
   if (out_f8) {
     a.out_f8 = out_f8;
     a.f8_scale = n.f8_scale + f8_slot;
@@ -745,20 +751,33 @@ static int gn_fwd(Net& n, GNL& g, const float* z, int N, int HW, float* out, boo
   return launch_gn_apply(a, N, HW, g.C, s);
 }
 
-// GroupNorm backward into n.dzop (op dtype). relu_y: the output of the ReLU that followed
-// the normalisation (its mask is applied to dy here); g_out receives the masked gradient.
+// GroupNorm backward into n.dzop (op dtype). The ReLU that followed the normalisation, if
+// any: Relu::from_z when nothing was added in between (its mask is recomputed from z), else
+// its output y (and the bits y > 0 where they were stored). Its mask is applied to dy here;
+// g_out receives the masked gradient.
+struct Relu {
+  const float* y = nullptr;
+  const uint8_t* pos = nullptr;
+  bool from_z = false;
+};
 static int gn_bwd(Net& n, GNL& g, const float* dy, const float* z, int N, int HW, bool first,
-                  cudaStream_t s, const float* relu_y = nullptr, float* g_out = nullptr) {
+                  cudaStream_t s, const Relu& relu = Relu(), float* g_out = nullptr) {
   GNBack b{};
-  b.dy = dy; b.relu_y = relu_y; b.g_out = g_out;
+  b.dy = dy; b.relu_y = relu.y; b.pos = relu.pos; b.g_out = g_out;
   b.z = z; b.mean = g.mean; b.rstd = g.rstd; b.gamma = n.params + g.g_off;
+  b.relu_from_z = relu.from_z ? 1 : 0; b.beta = n.params + g.b_off;
   b.m1 = n.gn_m1; b.m2 = n.gn_m2;
   b.dzop = n.dzop; b.op_bf16 = n.bf;
   b.dgamma_part = n.gnp_g; b.dbeta_part = n.gnp_b;
-  DDPPO_TRY(launch_gn_bwd(b, N, HW, g.C, n.gnw, s));
+  DDPPO_TRY(launch_gn_bwd(b, N, HW, g.C, n.gnw, n.gws.err, s));
   DDPPO_TRY(launch_colsum2(n.gnp_g, n.gnp_b, N, g.C, g.C, n.grad + g.g_off, n.grad + g.b_off,
                            !first, s));
   return DDPPO_OK;
+}
+static Relu relu_from_z() {
+  Relu r;
+  r.from_z = true;
+  return r;
 }
 
 static GConv gconv_of(const GConvL& g, int N) {
@@ -815,13 +834,13 @@ static int sx_block_bwd(Net& n, SxL& X, int N, const float* x, const __nv_bfloat
   DDPPO_TRY(launch_se_bwd(e, gcur, gcur, gA, !first, s));
   DDPPO_TRY(gn_bwd(n, X.n3, gA, X.c3.z, N, X.HW, first, s));
   DDPPO_TRY(conv_bwd(n, X.c3, X.n2.out, false, N, n.dzop, gB, false, first, s, X.n2.out_bf));
-  DDPPO_TRY(gn_bwd(n, X.n2, gB, X.c2.z, N, X.HW, first, s, X.n2.out));
+  DDPPO_TRY(gn_bwd(n, X.n2, gB, X.c2.z, N, X.HW, first, s, relu_from_z()));
   const GConv gc = gconv_of(X.c2, N);
   const void* g_in = n.bf ? (const void*)X.n1.out_bf : (const void*)X.n1.out;
   DDPPO_TRY(launch_gconv_wgrad(gc, g_in, n.dzop, n.gw_part, n.gw_part_elems, n.gws.num_sms,
                                n.grad + X.c2.w_off, first ? 0.f : 1.f, n.bf, s));
   DDPPO_TRY(launch_gconv_dgrad(gc, n.dzop, X.c2.wg, gA, false, n.bf, s));
-  DDPPO_TRY(gn_bwd(n, X.n1, gA, X.c1.z, N, HWi, first, s, X.n1.out));
+  DDPPO_TRY(gn_bwd(n, X.n1, gA, X.c1.z, N, HWi, first, s, relu_from_z()));
   if (X.down) {
     DDPPO_TRY(conv_bwd(n, X.c1, x, false, N, n.dzop, gB, false, first, s, x_bf));
     DDPPO_TRY(gn_bwd(n, X.nd, gcur, X.d.z, N, X.HW, first, s));
@@ -895,10 +914,10 @@ static int encoder_fwd(Net& n, const void* obs, int N, void* featop_rows, cudaSt
     if (B.down) {
       DDPPO_TRY(conv_fwd(n, B.d, cur, false, N, B.d.z, false, s, cur_bf, cur_f8, cur_sc));
       DDPPO_TRY(gn_fwd(n, B.n2, B.c2.z, N, HW, B.y, true, nullptr, &B.nd, B.d.z, s, y_bf, y_f8,
-                       B.y_slot));
+                       B.y_slot, B.pos));
     } else {
       DDPPO_TRY(gn_fwd(n, B.n2, B.c2.z, N, HW, B.y, true, cur, nullptr, nullptr, s, y_bf, y_f8,
-                       B.y_slot));
+                       B.y_slot, B.pos));
     }
     cur = B.y;
     cur_bf = y_bf;
@@ -931,7 +950,7 @@ static int encoder_bwd(Net& n, const void* obs, int N, const float* dfeat_rows, 
     return DDPPO_OK;
   }
   // compression conv
-  DDPPO_TRY(gn_bwd(n, n.cmp_n, dfeat_rows, n.cmp.z, N, n.featHW, first, s, n.cmp_n.out));
+  DDPPO_TRY(gn_bwd(n, n.cmp_n, dfeat_rows, n.cmp.z, N, n.featHW, first, s, relu_from_z()));
   const float* last_y = n.sx.empty() ? n.blocks[7].y : n.sx.back().y;
   const __nv_bfloat16* last_bf = n.sx.empty() ? n.blocks[7].y_bf : n.sx.back().y_bf;
   DDPPO_TRY(conv_bwd(n, n.cmp, last_y, false, N, n.dzop, n.g1, false, first, s, last_bf));
@@ -951,12 +970,15 @@ static int encoder_bwd(Net& n, const void* obs, int N, const float* dfeat_rows, 
     const __nv_bfloat16* xin_bf = bi > 0 ? n.blocks[bi - 1].y_bf : n.pool_bf;
     // the ReLU after the sum masks gcur; with an identity skip the masked gradient is
     // kept (written back in place) and the first conv's input gradient accumulates onto it
-    DDPPO_TRY(gn_bwd(n, B.n2, gcur, B.c2.z, N, HW, first, s, B.y, B.down ? nullptr : gcur));
+    Relu relu;
+    relu.y = B.y;
+    relu.pos = B.pos;
+    DDPPO_TRY(gn_bwd(n, B.n2, gcur, B.c2.z, N, HW, first, s, relu, B.down ? nullptr : gcur));
     DDPPO_TRY(conv_bwd(n, B.c2, B.n1.out, false, N, n.dzop, gA, false, first, s, B.n1.out_bf));
-    DDPPO_TRY(gn_bwd(n, B.n1, gA, B.c1.z, N, HW, first, s, B.n1.out));
+    DDPPO_TRY(gn_bwd(n, B.n1, gA, B.c1.z, N, HW, first, s, relu_from_z()));
     if (B.down) {
       DDPPO_TRY(conv_bwd(n, B.c1, xin, false, N, n.dzop, gB, false, first, s, xin_bf));
-      DDPPO_TRY(gn_bwd(n, B.nd, gcur, B.d.z, N, HW, first, s, B.y));
+      DDPPO_TRY(gn_bwd(n, B.nd, gcur, B.d.z, N, HW, first, s, relu));
       DDPPO_TRY(conv_bwd(n, B.d, xin, false, N, n.dzop, gB, true, first, s, xin_bf));
       float* t = gcur; gcur = gB; gB = t;
     } else {
@@ -965,25 +987,10 @@ static int encoder_bwd(Net& n, const void* obs, int N, const float* dfeat_rows, 
   }
   // max pool, stem GN + ReLU, stem conv (no input gradient)
   ConvL& st = n.stem;
-  if (st.cout % 4 == 0) {
-    // the max-pool gradient scattered once; the GroupNorm backward recomputes the ReLU
-    // mask from z (the full-resolution activation was never stored)
-    DDPPO_TRY(launch_maxpool_bwd(gcur, n.pool_arg, N, st.Ho, st.Wo, st.cout, gA, s));
-    GNBack b{};
-    b.dy = gA;
-    b.z = st.z; b.mean = n.stem_n.mean; b.rstd = n.stem_n.rstd;
-    b.gamma = n.params + n.stem_n.g_off; b.beta = n.params + n.stem_n.b_off;
-    b.relu_from_z = 1;
-    b.m1 = n.gn_m1; b.m2 = n.gn_m2;
-    b.dzop = n.dzop; b.op_bf16 = n.bf;
-    b.dgamma_part = n.gnp_g; b.dbeta_part = n.gnp_b;
-    DDPPO_TRY(launch_gn_bwd(b, N, st.Ho * st.Wo, st.cout, n.gnw, s));
-    DDPPO_TRY(launch_colsum2(n.gnp_g, n.gnp_b, N, st.cout, st.cout, n.grad + n.stem_n.g_off,
-                             n.grad + n.stem_n.b_off, !first, s));
-  } else {
-    DDPPO_TRY(launch_maxpool_bwd(gcur, n.pool_arg, N, st.Ho, st.Wo, st.cout, gA, s));
-    DDPPO_TRY(gn_bwd(n, n.stem_n, gA, st.z, N, st.Ho * st.Wo, first, s, n.stem_n.out));
-  }
+  // the max-pool gradient scattered once; the GroupNorm backward recomputes the ReLU mask
+  // from z (the full-resolution activation need not be stored)
+  DDPPO_TRY(launch_maxpool_bwd(gcur, n.pool_arg, N, st.Ho, st.Wo, st.cout, gA, s));
+  DDPPO_TRY(gn_bwd(n, n.stem_n, gA, st.z, N, st.Ho * st.Wo, first, s, relu_from_z()));
   DDPPO_TRY(conv_bwd(n, st, obs, n.bf, N, n.dzop, nullptr, false, first, s));
   return DDPPO_OK;
 }

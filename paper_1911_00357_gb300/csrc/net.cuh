@@ -46,6 +46,7 @@ struct BlockL {
   bool down = false;
   float* y = nullptr;     // block output [NC, Ho, Wo, cout]
   __nv_bfloat16* y_bf = nullptr;  // its bf16 copy (BF16 form)
+  uint8_t* pos = nullptr;         // [NC, Ho, Wo, cout / 4] bits y > 0 (null when cout % 4)
   uint8_t* y_f8 = nullptr;        // [E, Ho, Wo, cout] its E4M3 copy (FP8 inference)
   int y_slot = -1;
 };

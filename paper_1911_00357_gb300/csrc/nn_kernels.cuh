@@ -43,23 +43,27 @@ struct GNApply {
   const float* z; const float* mean; const float* rstd; const float* gamma; const float* beta;
   const float* resid;  // or null
   const float* zd; const float* mean_d; const float* rstd_d; const float* gamma_d; const float* beta_d;
-  float* out; int relu;
+  float* out; int relu;   // out null: only the other forms are stored
   __nv_bfloat16* out_bf;  // optional bf16 copy of out (the next convolution's TMA operand)
   // optional E4M3 copy of out for FP8 inference: e4m3(out / *f8_scale), saturating, and
   // the largest |out| folded into *f8_amax (float bits; a max, so the order is irrelevant)
   uint8_t* out_f8; const float* f8_scale; unsigned* f8_amax;
+  // optional: one byte per 4 channels, bit v set where channel v of out is > 0 (the ReLU's
+  // mask for the backward, a sixteenth of reading out again); C % 4 == 0
+  uint8_t* pos;
 };
 int launch_gn_apply(const GNApply& a, int N, int HW, int C, cudaStream_t s);
-// statistics and normalisation in one cooperative launch: a.mean/a.rstd (and a.mean_d /
-// a.rstd_d with zd) receive the statistics, out as launch_gn_apply. Sets *launched = false,
-// launching nothing, when an image takes one block (small images: the two launches are
-// faster), when the grid cannot be resident at once (many images) or w has no departure
-// counters; the caller then runs launch_gn_stats + launch_gn_apply. err: the sticky status
-// word (timeout flag on a barrier run-out).
+// statistics and normalisation in one launch: a.mean/a.rstd (and a.mean_d / a.rstd_d with
+// zd) receive the statistics, out as launch_gn_apply. Images summed by one block each:
+// slices of an image's channels staged in shared memory, one block each. Larger images: a
+// cooperative launch. Sets *launched = false, launching nothing, when neither form covers
+// the shape (grid not resident at once, slice too large for shared memory); the caller then
+// runs launch_gn_stats + launch_gn_apply, with the same bits. err: the sticky status word
+// (timeout flag on a barrier run-out).
 int launch_gn_fused(const GNApply& a, int N, int HW, int C, float eps, const GnScratch& w,
                     int32_t* err, cudaStream_t s, bool* launched);
-// GroupNorm backward. g = dy, masked by (relu_y > 0) when relu_y is given (the ReLU that
-// followed the normalisation); g_out (optional, with relu_y) receives g.
+// GroupNorm backward. g = dy, masked by (relu_y > 0) when relu_y or pos is given (the ReLU
+// that followed the normalisation); g_out (optional, with relu_y or pos) receives g.
 //   dz = rstd (g gamma - m1 - xhat m2), m1 / m2 the group means of gamma g and gamma g xhat;
 //   dgamma_part[n, c] = sum g xhat, dbeta_part[n, c] = sum g (per image).
 // m1, m2: [N, C/2] scratch. dz32 (fp32) and dzop (op dtype) each optional.
@@ -72,8 +76,12 @@ struct GNBack {
   // optional: the ReLU after the normalisation was not stored; its mask is recomputed
   // from z (relu_y unused, beta = the GroupNorm shift)
   int relu_from_z; const float* beta;
+  // optional: relu_y > 0 as GNApply's pos bits (read instead of relu_y; C % 4 == 0)
+  const uint8_t* pos;
 };
-int launch_gn_bwd(const GNBack& b, int N, int HW, int C, const GnScratch& w, cudaStream_t s);
+// err: the sticky status word (timeout flag when a bounded copy wait runs out).
+int launch_gn_bwd(const GNBack& b, int N, int HW, int C, const GnScratch& w, int32_t* err,
+                  cudaStream_t s);
 // GroupNorm apply + ReLU + 3x3 / stride-2 / pad-1 max pool in one pass: pool (fp32),
 // pool_bf (bf16, optional), arg (argmax tap) of [N, Hq, Wq, C]; the full-resolution
 // activation is not written. C % 4 == 0.
