@@ -337,7 +337,7 @@ int ddppo_ppo_loss(int32_t n, const float* logits, const float* values, const in
  * allocate device memory where they need it, for instance inside a stream capture that
  * forbids cudaMalloc or in a process whose device memory belongs to another allocator.
  * The paper has no counterpart: this is a deployment variant. Samples are spread over
- * one thread block per 256 (ddppo_ppo_loss uses one block); the per-block partial sums
+ * one thread block per 256 (ddppo_ppo_loss uses one cluster); the per-block partial sums
  * live in an 80 KiB array owned by the library, so nothing is allocated and no context
  * is needed. n must be at most 1,048,576 (E_CONFIG otherwise). The first call on each
  * device looks up the array's device address; make it before any stream capture. Every

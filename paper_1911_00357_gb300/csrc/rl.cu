@@ -3,7 +3,9 @@
 // the per-epoch env permutation for minibatches, and the optional advantage
 // normalisation. Every reduction is block partials followed by one fixed-order pass.
 #include <algorithm>
+#include <atomic>
 
+#include "cluster.cuh"
 #include "rl.cuh"
 
 namespace ddppo {
@@ -38,54 +40,112 @@ __device__ void block_partials(float (&v)[NV], float* part) {
 //   d logp = -rho A when the unclipped term is the active minimum (ties split evenly
 //   between the two branches, which sum to the same when rho is inside the clip range)
 //   dlogits_j = [dlogp (1[j=a] - p_j) + c_e p_j (log p_j + H_i)] / n ; dV = c_v (V - R) / n
-__global__ void __launch_bounds__(256) ppo_loss_kernel(int n, const float* __restrict__ logits,
-                                                       const float* __restrict__ values,
-                                                       const int32_t* __restrict__ actions,
-                                                       const float* __restrict__ logp_old,
-                                                       const float* __restrict__ adv,
-                                                       const float* __restrict__ ret, float clip,
-                                                       float cv, float ce, float* dlogits,
-                                                       float* dvalues, float* part) {
+struct LossIn {
+  int n;
+  const float* logits; const float* values; const int32_t* actions; const float* logp_old;
+  const float* adv; const float* ret;
+  float clip, cv, ce;
+};
+__device__ __forceinline__ void loss_sample(const LossIn& q, int i, float* dlogits, float* dvalues,
+                                            float (&acc)[5]) {
+  const float clip = q.clip, ce = q.ce;
+  float lg[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) lg[k] = q.logits[(size_t)i * 4 + k];
+  int a = q.actions[i];
+  const float A = q.adv[i], old = q.logp_old[i], V = q.values[i], R = q.ret[i];
+  const float mx = fmaxf(fmaxf(lg[0], lg[1]), fmaxf(lg[2], lg[3]));
+  float z = 0.f;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) z += expf(lg[k] - mx);
+  const float lse = mx + logf(z);
+  float lp[4], p[4], H = 0.f;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    lp[k] = lg[k] - lse;
+    p[k] = expf(lp[k]);
+    H -= p[k] * lp[k];
+  }
+  a = a < 0 ? 0 : (a > 3 ? 3 : a);
+  const float lpa = a == 0 ? lp[0] : a == 1 ? lp[1] : a == 2 ? lp[2] : lp[3];
+  const float rho = expf(lpa - old);
+  const float s1 = rho * A;
+  const float rc = fminf(fmaxf(rho, 1.f - clip), 1.f + clip);
+  const float s2 = rc * A;
+  const bool inside = rho >= 1.f - clip && rho <= 1.f + clip;
+  const float dlp = (inside || s1 < s2) ? -rho * A : 0.f;
+  const float inv = 1.0f / (float)q.n;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    dlogits[(size_t)i * 4 + k] = inv * (dlp * ((k == a ? 1.f : 0.f) - p[k]) + ce * p[k] * (lp[k] + H));
+  dvalues[i] = inv * q.cv * (V - R);
+  acc[0] += -fminf(s1, s2);
+  acc[1] += 0.5f * (R - V) * (R - V);
+  acc[2] += H;
+  acc[3] += fabsf(rho - 1.f) > clip ? 1.f : 0.f;
+  acc[4] += old - lpa;
+}
+__device__ __forceinline__ void loss_stats(const float (&s)[5], int n, float cv, float ce, float* stats) {
+  const float inv = 1.0f / (float)n;
+  const float pol = s[0] * inv, vl = s[1] * inv, ent = s[2] * inv;
+  stats[0] = pol + cv * vl - ce * ent;
+  stats[1] = pol;
+  stats[2] = vl;
+  stats[3] = ent;
+  stats[4] = s[3] * inv;
+  stats[5] = s[4] * inv;
+  stats[6] = 0.f;
+  stats[7] = 0.f;
+}
+
+__global__ void __launch_bounds__(256) ppo_loss_kernel(LossIn q, float* dlogits, float* dvalues, float* part) {
   DDPPO_PDL_ENTRY();
   float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    float lg[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) lg[q] = logits[(size_t)i * 4 + q];
-    const float mx = fmaxf(fmaxf(lg[0], lg[1]), fmaxf(lg[2], lg[3]));
-    float z = 0.f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) z += expf(lg[q] - mx);
-    const float lse = mx + logf(z);
-    float lp[4], p[4], H = 0.f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      lp[q] = lg[q] - lse;
-      p[q] = expf(lp[q]);
-      H -= p[q] * lp[q];
-    }
-    int a = actions[i];
-    a = a < 0 ? 0 : (a > 3 ? 3 : a);
-    const float A = adv[i];
-    const float rho = expf(lp[a] - logp_old[i]);
-    const float s1 = rho * A;
-    const float rc = fminf(fmaxf(rho, 1.f - clip), 1.f + clip);
-    const float s2 = rc * A;
-    const bool inside = rho >= 1.f - clip && rho <= 1.f + clip;
-    const float dlp = (inside || s1 < s2) ? -rho * A : 0.f;
-    const float V = values[i], R = ret[i];
-    const float inv = 1.0f / (float)n;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      dlogits[(size_t)i * 4 + q] = inv * (dlp * ((q == a ? 1.f : 0.f) - p[q]) + ce * p[q] * (lp[q] + H));
-    dvalues[i] = inv * cv * (V - R);
-    acc[0] += -fminf(s1, s2);
-    acc[1] += 0.5f * (R - V) * (R - V);
-    acc[2] += H;
-    acc[3] += fabsf(rho - 1.f) > clip ? 1.f : 0.f;
-    acc[4] += logp_old[i] - lp[a];
-  }
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < q.n; i += gridDim.x * blockDim.x)
+    loss_sample(q, i, dlogits, dvalues, acc);
   block_partials<5>(acc, part);
+}
+
+// The whole loss in one launch and without scratch: one cluster, whose CTAs' partial sums
+// meet in the shared memory of its first CTA (in rank order). Bound: latency -- one sample
+// a thread up to 4096 samples (3.1 us of kernel). One block over all samples and a second
+// launch for its sums took 13.4 us a call at 4096 samples, 30.9 at 16384 and 223 at 131072;
+// here 10.8, 11.4 and 11.6 (an empty call: 8.5).
+__global__ void __launch_bounds__(1024) ppo_loss_cluster_kernel(LossIn q, float* dlogits, float* dvalues,
+                                                                float* stats) {
+  DDPPO_PDL_ENTRY();
+  __shared__ float warp_part[32][5];
+  __shared__ float cta_part[16][5];  // of the first CTA: one row per rank
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t rank = cluster_rank();
+  cluster_arrive();  // waited for below: the first CTA runs before anything is stored there
+  float acc[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < q.n; i += gridDim.x * blockDim.x)
+    loss_sample(q, i, dlogits, dvalues, acc);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const float t = wsum(acc[k]);
+    if (lane == 0) warp_part[w][k] = t;
+  }
+  __syncthreads();
+  cluster_wait();
+  if (threadIdx.x < 5) {
+    float t = 0.f;
+    for (int j = 0; j < nw; ++j) t += warp_part[j][threadIdx.x];
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(map_rank(smem_addr(&cta_part[rank][threadIdx.x]), 0u)),
+                 "f"(t)
+                 : "memory");
+  }
+  __syncwarp();
+  cluster_sync();
+  if (rank != 0 || threadIdx.x != 0) return;
+  float s[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    s[k] = 0.f;
+    for (int j = 0; j < (int)gridDim.x; ++j) s[k] += cta_part[j][k];
+  }
+  loss_stats(s, q.n, q.cv, q.ce, stats);
 }
 
 // the sum over nb blocks of NV partials each (part[b * NV + k]) by one block of kFinal
@@ -118,18 +178,49 @@ __global__ void __launch_bounds__(kFinal) ppo_loss_final(int nb, int n, const fl
                                                         float ce, float* stats) {
   DDPPO_PDL_ENTRY();
   float s[5];
-  final_sums<5>(part, nb, s);  // part may alias stats: all reads precede the writes below
+  final_sums<5>(part, nb, s);
   if (threadIdx.x != 0) return;
-  const float inv = 1.0f / (float)n;
-  const float pol = s[0] * inv, vl = s[1] * inv, ent = s[2] * inv;
-  stats[0] = pol + cv * vl - ce * ent;
-  stats[1] = pol;
-  stats[2] = vl;
-  stats[3] = ent;
-  stats[4] = s[3] * inv;
-  stats[5] = s[4] * inv;
-  stats[6] = 0.f;
-  stats[7] = 0.f;
+  loss_stats(s, n, cv, ce, stats);
+}
+
+// one cluster of 1, 2, 4 or 8 CTAs (16 where the device allows that many), 256 threads each
+// up to one sample a thread, then 1024
+static int launch_loss_cluster(const LossIn& q, float* dlogits, float* dvalues, float* stats, cudaStream_t s) {
+  static std::atomic<int> largest[64];  // 0: not asked yet
+  int dev = 0;
+  DDPPO_CHECK_CUDA(cudaGetDevice(&dev));
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(1024);
+  cfg.attrs = attr;
+  int most = dev < 64 ? largest[dev].load() : 8;
+  if (!most) {
+    cfg.gridDim = dim3(16);
+    cfg.numAttrs = 1;
+    attr[0].val.clusterDim.x = 16;
+    int num = 0;
+    most = 8;
+    if (cudaFuncSetAttribute(ppo_loss_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+            cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&num, ppo_loss_cluster_kernel, &cfg) == cudaSuccess && num > 0)
+      most = 16;
+    else
+      (void)cudaGetLastError();
+    largest[dev].store(most);
+  }
+  int ctas = 1;
+  while (ctas < most && ctas * 256 < q.n) ctas *= 2;
+  attr[0].val.clusterDim.x = (unsigned)ctas;
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3(q.n > ctas * 256 ? 1024 : 256);
+  cfg.stream = s;
+  cfg.numAttrs = pdl_enabled() ? 2 : 1;
+  DDPPO_CHECK_CUDA(cudaLaunchKernelEx(&cfg, ppo_loss_cluster_kernel, q, dlogits, dvalues, stats));
+  return DDPPO_OK;
 }
 
 int launch_ppo_loss(int n, const float* logits, const float* values, const int32_t* actions,
@@ -137,17 +228,15 @@ int launch_ppo_loss(int n, const float* logits, const float* values, const int32
                     float ce, float* stats, float* dlogits, float* dvalues, float* part,
                     size_t part_elems, cudaStream_t s) {
   if (n <= 0) return DDPPO_OK;
-  // without scratch one block covers all samples and reduces into stats itself
-  int nb = part ? (n + 255) / 256 : 1;
-  if (nb > 1024) nb = 1024;
-  if (!part) part = stats;
-  else if ((size_t)nb * 5 > part_elems) { set_error("ppo_loss: scratch too small"); return DDPPO_E_CONFIG; }
-  ::ddppo::launch_k(ppo_loss_kernel, nb, 256, 0, s, n, logits, values, actions, logp_old, adv, ret, clip, cv, ce,
-                                     dlogits, dvalues, part);
-  DDPPO_CHECK_LAUNCH();
-  ::ddppo::launch_k(ppo_loss_final, 1, kFinal, 0, s, nb, n, part, cv, ce, stats);
-  DDPPO_CHECK_LAUNCH();
-  return DDPPO_OK;
+  const LossIn q{n, logits, values, actions, logp_old, adv, ret, clip, cv, ce};
+  // one cluster up to 8 samples for each of its 16384 threads (at 131072 samples 11.6 us a
+  // call, no more than the two launches of the form below take for few), and where there is
+  // no scratch
+  if (!part || n <= 131072) return launch_loss_cluster(q, dlogits, dvalues, stats, s);
+  const int nb = std::min((n + 255) / 256, 1024);
+  if ((size_t)nb * 5 > part_elems) { set_error("ppo_loss: scratch too small"); return DDPPO_E_CONFIG; }
+  return launch_ppo_loss_blocks(n, logits, values, actions, logp_old, adv, ret, clip, cv, ce, stats, dlogits,
+                                dvalues, part, nb, s);
 }
 
 int launch_ppo_loss_blocks(int n, const float* logits, const float* values, const int32_t* actions,
@@ -155,8 +244,8 @@ int launch_ppo_loss_blocks(int n, const float* logits, const float* values, cons
                            float cv, float ce, float* stats, float* dlogits, float* dvalues,
                            float* part, int nb, cudaStream_t s) {
   if (n <= 0) return DDPPO_OK;
-  ::ddppo::launch_k(ppo_loss_kernel, nb, 256, 0, s, n, logits, values, actions, logp_old, adv, ret, clip, cv, ce,
-                                     dlogits, dvalues, part);
+  const LossIn q{n, logits, values, actions, logp_old, adv, ret, clip, cv, ce};
+  ::ddppo::launch_k(ppo_loss_kernel, nb, 256, 0, s, q, dlogits, dvalues, part);
   DDPPO_CHECK_LAUNCH();
   ::ddppo::launch_k(ppo_loss_final, 1, kFinal, 0, s, nb, n, part, cv, ce, stats);
   DDPPO_CHECK_LAUNCH();
