@@ -67,6 +67,27 @@ inline void launch_k(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cud
   (void)cudaLaunchKernelEx(&cfg, kern, static_cast<A&&>(args)...);  // checked by the caller
 }
 
+// the same with thread-block clusters of `cluster` CTAs (at most 8: the portable size)
+template <typename... P, typename... A>
+inline void launch_cluster_k(void (*kern)(P...), dim3 grid, dim3 block, dim3 cluster, size_t smem, cudaStream_t s,
+                             A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster.x;
+  attr[0].val.clusterDim.y = cluster.y;
+  attr[0].val.clusterDim.z = cluster.z;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl_enabled() ? 2 : 1;
+  (void)cudaLaunchKernelEx(&cfg, kern, static_cast<A&&>(args)...);  // checked by the caller
+}
+
 // sticky device error word: bit flags
 enum : int32_t { ERRF_BOUNDS = 1, ERRF_TIMEOUT = 2, ERRF_RESET = 4 };
 enum : int { TASK_POINTGOAL = 0, TASK_FLEE = 1, TASK_EXPLORE = 2 };

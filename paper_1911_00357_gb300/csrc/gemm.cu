@@ -5,137 +5,297 @@
 
 namespace ddppo {
 
-template <typename T>
-__device__ __forceinline__ float ld_op(const T* p);
-template <>
-__device__ __forceinline__ float ld_op<float>(const float* p) { return __ldg(p); }
-template <>
-__device__ __forceinline__ float ld_op<__nv_bfloat16>(const __nv_bfloat16* p) {
-  return __bfloat162float(*p);
+// 4 neighbouring operands, element i present where i < n (vec: 4-element aligned rows)
+__device__ __forceinline__ float4 ld4(const float* p, int n, bool vec) {
+  if (vec && n >= 4) return __ldg((const float4*)p);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (n > 0) v.x = __ldg(p);
+  if (n > 1) v.y = __ldg(p + 1);
+  if (n > 2) v.z = __ldg(p + 2);
+  if (n > 3) v.w = __ldg(p + 3);
+  return v;
+}
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p, int n, bool vec) {
+  if (vec && n >= 4) {
+    const uint2 u = __ldg((const uint2*)p);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                       __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+  }
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (n > 0) v.x = __bfloat162float(p[0]);
+  if (n > 1) v.y = __bfloat162float(p[1]);
+  if (n > 2) v.z = __bfloat162float(p[2]);
+  if (n > 3) v.w = __bfloat162float(p[3]);
+  return v;
 }
 
-constexpr int SB_M = 64, SB_N = 64, SB_K = 16;
+constexpr int SB_K = 16;
+constexpr int kSplitSteps = 2;  // steps of SB_K a K split has at least
 
-// 256 threads; thread (tx, ty) owns rows ty + 16 i and columns tx + 16 j, i, j < 4.
-template <typename T>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K, const T* __restrict__ A,
-                                                        int lda, const T* __restrict__ B, int ldb,
-                                                        float* __restrict__ C, int ldc, int c_bf16,
-                                                        float beta, const float* __restrict__ bias,
-                                                        int relu, int kchunk,
-                                                        float* __restrict__ partial, int a_t,
-                                                        int b_t) {
-  DDPPO_PDL_ENTRY();
-  __shared__ float As[SB_K][SB_M + 4];
-  __shared__ float Bs[SB_K][SB_N + 4];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.x * SB_M, n0 = blockIdx.y * SB_N;  // M tiles on x: M can exceed 65535*64
-  const int kbeg = blockIdx.z * kchunk, kend = min(K, kbeg + kchunk);
-  float acc[4][4] = {};
-  const int lr = tid >> 2, lk = (tid & 3) * 4;  // loader: row lr, k lk..lk+3
-  for (int k0 = kbeg; k0 < kend; k0 += SB_K) {
+// One operand's BR x SB_K tile: registers while the previous tile is multiplied, then shared
+// memory [k][row]. K-contiguous rows are transposed on the way; rows stored [K][R] are not.
+template <int BR, typename T>
+struct SimtTile {
+  static constexpr int kUnits = BR * SB_K / 4;        // groups of 4 elements
+  static constexpr int kPer = (kUnits + 255) / 256;   // per thread
+  float4 v[kPer];
+  __device__ __forceinline__ void load(const T* p, int ld, int r0, int R, int k0, int kend, bool t, bool vec) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int k = k0 + lk + q;
-      const int m = m0 + lr, n = n0 + lr;
-      As[lk + q][lr] = (m < M && k < kend)
-                           ? ld_op(A + (a_t ? (size_t)k * lda + m : (size_t)m * lda + k)) : 0.f;
-      Bs[lk + q][lr] = (n < N && k < kend)
-                           ? ld_op(B + (b_t ? (size_t)k * ldb + n : (size_t)n * ldb + k)) : 0.f;
+    for (int i = 0; i < kPer; ++i) {
+      const int u = threadIdx.x + 256 * i;
+      v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (kUnits % 256 && u >= kUnits) continue;
+      if (t) {
+        const int k = k0 + u / (BR / 4), r = r0 + u % (BR / 4) * 4;
+        if (k < kend) v[i] = ld4(p + (size_t)k * ld + r, R - r, vec);
+      } else {
+        const int r = r0 + (u >> 2), k = k0 + (u & 3) * 4;
+        if (r < R) v[i] = ld4(p + (size_t)r * ld + k, kend - k, vec);
+      }
     }
-    __syncthreads();
+  }
+  __device__ __forceinline__ void store(float (*sh)[BR + 4], bool t) const {
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const int u = threadIdx.x + 256 * i;
+      if (kUnits % 256 && u >= kUnits) continue;
+      if (t) {
+        *(float4*)&sh[u / (BR / 4)][u % (BR / 4) * 4] = v[i];
+      } else {
+        const int r = u >> 2, k = (u & 3) * 4;
+        sh[k][r] = v[i].x;
+        sh[k + 1][r] = v[i].y;
+        sh[k + 2][r] = v[i].z;
+        sh[k + 3][r] = v[i].w;
+      }
+    }
+  }
+};
+
+enum { SIMT_VEC_A = 1, SIMT_VEC_B = 2, SIMT_VEC_C = 4 };
+struct SimtArgs {
+  int M, N, K, lda, ldb, ldc, c_bf16, relu, kchunk, a_t, b_t, vec;
+  const void* A;
+  const void* B;
+  float* C;
+  float beta;
+  const float* bias;
+  float* partial;
+};
+
+// C tile BM x BN a CTA; a thread owns TM/4 groups of 4 rows (BM / (TM/4) apart) by 4
+// neighbouring columns, so an operand read is one 16-byte shared load and TM x 4 FMAs use
+// TM/4 + 1 of them. Each output's sum runs over k in ascending order, one FMA a step.
+// Bound: FP32 FMA issue; the next tile's global loads are in flight while this one is
+// multiplied (two shared buffers, one barrier a tile). A 64x64 tile with scalar loads and
+// 8 shared loads per 16 FMAs took 29 us a launch over the 60 GEMMs of the small FP32 update
+// (3.3 ms of update in all); this form 8.7.
+template <int BM, int BN, int TM, typename T>
+__global__ void __launch_bounds__(256) gemm_simt_kernel(const SimtArgs q) {
+  DDPPO_PDL_ENTRY();
+  constexpr int TX = BN / 4, G = TM / 4, MS = BM / G;
+  static_assert(TX * (BM / TM) == 256, "one micro-tile a thread");
+  __shared__ __align__(16) float As[2][SB_K][BM + 4];
+  __shared__ __align__(16) float Bs[2][SB_K][BN + 4];
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  const int M = q.M, N = q.N;
+  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;  // M tiles on x: M can exceed 65535 tiles
+  const int kbeg = blockIdx.z * q.kchunk, kend = min(q.K, kbeg + q.kchunk);
+  const T* A = (const T*)q.A;
+  const T* B = (const T*)q.B;
+  const bool va = q.vec & SIMT_VEC_A, vb = q.vec & SIMT_VEC_B, at = q.a_t, bt = q.b_t;
+  float acc[TM][4] = {};
+  SimtTile<BM, T> ta;
+  SimtTile<BN, T> tb;
+  ta.load(A, q.lda, m0, M, kbeg, kend, at, va);
+  tb.load(B, q.ldb, n0, N, kbeg, kend, bt, vb);
+  int buf = 0;
+  for (int k0 = kbeg; k0 < kend; k0 += SB_K, buf ^= 1) {
+    ta.store(As[buf], at);
+    tb.store(Bs[buf], bt);
+    __syncthreads();  // also: every thread is done with the other buffer's previous tile
+    if (k0 + SB_K < kend) {
+      ta.load(A, q.lda, m0, M, k0 + SB_K, kend, at, va);
+      tb.load(B, q.ldb, n0, N, k0 + SB_K, kend, bt, vb);
+    }
 #pragma unroll
     for (int kk = 0; kk < SB_K; ++kk) {
-      float a[4], b[4];
+      const float4 b = *(const float4*)&Bs[buf][kk][tx * 4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+      for (int g = 0; g < G; ++g) {
+        const float4 a = *(const float4*)&As[buf][kk][g * MS + ty * 4];
+        const float av[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int i = 0; i < 4; ++i) {
+          float* c = acc[g * 4 + i];
+          c[0] = fmaf(av[i], b.x, c[0]);
+          c[1] = fmaf(av[i], b.y, c[1]);
+          c[2] = fmaf(av[i], b.z, c[2]);
+          c[3] = fmaf(av[i], b.w, c[3]);
+        }
+      }
     }
-    __syncthreads();
   }
+  const int n = n0 + tx * 4;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty + 16 * i;
+  for (int i = 0; i < TM; ++i) {
+    const int m = m0 + i / 4 * MS + ty * 4 + i % 4;
     if (m >= M) continue;
+    if (q.partial) {
+      float* p = q.partial + ((size_t)blockIdx.z * M + m) * N + n;
+      if ((q.vec & SIMT_VEC_C) && n + 3 < N) {
+        *(float4*)p = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (n + j < N) p[j] = acc[i][j];
+      }
+      continue;
+    }
+    const size_t o = (size_t)m * q.ldc + n;
+    float v[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx + 16 * j;
-      if (n >= N) continue;
-      if (partial) {
-        partial[((size_t)blockIdx.z * M + m) * N + n] = acc[i][j];
-        continue;
+      v[j] = acc[i][j];
+      if (n + j >= N) continue;
+      if (q.beta != 0.f) v[j] += q.beta * q.C[o + j];
+      if (q.bias) v[j] += q.bias[n + j];
+      if (q.relu) v[j] = fmaxf(v[j], 0.f);
+    }
+    if ((q.vec & SIMT_VEC_C) && n + 3 < N) {
+      *(float4*)(q.C + o) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (n + j >= N) continue;
+        if (q.c_bf16) ((__nv_bfloat16*)q.C)[o + j] = __float2bfloat16_rn(v[j]);
+        else q.C[o + j] = v[j];
       }
-      float v = acc[i][j];
-      if (beta != 0.f) v += beta * C[(size_t)m * ldc + n];
-      if (bias) v += bias[n];
-      if (relu) v = fmaxf(v, 0.f);
-      if (c_bf16) ((__nv_bfloat16*)C)[(size_t)m * ldc + n] = __float2bfloat16_rn(v);
-      else C[(size_t)m * ldc + n] = v;
     }
   }
 }
 
-// C = beta*C + sum_z partial[z] (+ bias) (ReLU), summed in split order.
-__global__ void splitk_reduce_kernel(int M, int N, int splits, const float* __restrict__ partial,
-                                     float* __restrict__ C, int ldc, int c_bf16, float beta,
-                                     const float* __restrict__ bias, int relu) {
+// C = beta*C + sum_z partial[z] (+ bias) (ReLU), summed in split order. V neighbouring
+// columns a thread: 1 for few outputs (latency: as many threads as there are outputs), 4 for
+// many (a quarter of the blocks). Several loads
+// in flight, added in order: at 64 frames the encoder's 12 reductions took 49 us a step with
+// one output a thread, 34 now; the FP32 update's 48 small ones 154 us in blocks of 256 and
+// dependent loads, 139 now.
+template <int V>
+__device__ __forceinline__ void add_partial(float (&v)[V], const float (&u)[V]) {
+#pragma unroll
+  for (int j = 0; j < V; ++j) v[j] += u[j];
+}
+template <int V>
+__device__ __forceinline__ void load_partial(float (&u)[V], const float* p) {
+  if constexpr (V == 4) {
+    const float4 t = *(const float4*)p;
+    u[0] = t.x; u[1] = t.y; u[2] = t.z; u[3] = t.w;
+  } else {
+    u[0] = *p;
+  }
+}
+template <int V>
+__global__ void __launch_bounds__(256) splitk_reduce_kernel(int M, int N, int splits,
+                                                            const float* __restrict__ partial,
+                                                            float* __restrict__ C, int ldc, int c_bf16,
+                                                            float beta, const float* __restrict__ bias,
+                                                            int relu) {
   DDPPO_PDL_ENTRY();
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)M * N) return;
+  const size_t idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * V, mn = (size_t)M * N;
+  if (idx >= mn) return;
   const int m = (int)(idx / N), n = (int)(idx % N);
-  float v = 0.f;
-  for (int z = 0; z < splits; ++z) v += partial[(size_t)z * M * N + idx];
-  if (beta != 0.f) v += beta * C[(size_t)m * ldc + n];
-  if (bias) v += bias[n];
-  if (relu) v = fmaxf(v, 0.f);
-  if (c_bf16) ((__nv_bfloat16*)C)[(size_t)m * ldc + n] = __float2bfloat16_rn(v);
-  else C[(size_t)m * ldc + n] = v;
+  const float* p = partial + idx;
+  float v[V] = {};
+  int z = 0;
+  constexpr int F = V == 4 ? 4 : 8;
+  for (; z + F <= splits; z += F, p += F * mn) {
+    float u[F][V];
+#pragma unroll
+    for (int i = 0; i < F; ++i) load_partial<V>(u[i], p + i * mn);
+#pragma unroll
+    for (int i = 0; i < F; ++i) add_partial<V>(v, u[i]);
+  }
+#pragma unroll 3
+  for (; z < splits; ++z, p += mn) {
+    float u[V];
+    load_partial<V>(u, p);
+    add_partial<V>(v, u);
+  }
+  const size_t o = (size_t)m * ldc + n;
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    if (beta != 0.f) v[j] += beta * C[o + j];
+    if (bias) v[j] += bias[n + j];
+    if (relu) v[j] = fmaxf(v[j], 0.f);
+    if (c_bf16) ((__nv_bfloat16*)C)[o + j] = __float2bfloat16_rn(v[j]);
+    else if (V == 1) C[o] = v[0];
+  }
+  if constexpr (V == 4)
+    if (!c_bf16) *(float4*)(C + o) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
-static int gemm_simt(const GemmDesc& d, bool op_bf16, const GemmWorkspace& ws, cudaStream_t s) {
-  const int gm = (d.M + SB_M - 1) / SB_M, gn = (d.N + SB_N - 1) / SB_N;
-  int splits = 1;
-  const int tiles = gm * gn;
-  const int target = 2 * ws.num_sms;
-  if (tiles < target && d.K >= 4 * SB_K * 8) {
-    splits = (target + tiles - 1) / tiles;
-    splits = min(splits, d.K / (SB_K * 8));
-    const size_t per = (size_t)d.M * d.N;
+// 4-element groups of a row are aligned for the vector load or store of `bytes` an element
+static bool rows_of_4(const void* p, int ld, int bytes) {
+  return ld % 4 == 0 && ((uintptr_t)p & (uintptr_t)(4 * bytes - 1)) == 0;
+}
+
+template <int BM, int BN, int TM>
+static void launch_simt(SimtArgs& q, bool op_bf16, const GemmWorkspace& ws, int& splits, cudaStream_t s) {
+  const int gm = (q.M + BM - 1) / BM, gn = (q.N + BN - 1) / BN;
+  const int tiles = gm * gn, target = 2 * ws.num_sms;
+  splits = 1;
+  // too few tiles for the chip: split K, at least two steps of SB_K a split (8 steps: 11.7
+  // us instead of 6.9 for the update's 64x64-tiled launches)
+  if (tiles < target && q.K >= 4 * SB_K * kSplitSteps) {
+    splits = min((target + tiles - 1) / tiles, q.K / (SB_K * kSplitSteps));
+    const size_t per = (size_t)q.M * q.N;
     if (per > 0) splits = (int)min((size_t)splits, ws.partial_elems / per);
     if (splits < 2) splits = 1;
   }
-  int kchunk = (d.K + splits - 1) / splits;
-  kchunk = (kchunk + SB_K - 1) / SB_K * SB_K;
-  splits = (d.K + kchunk - 1) / kchunk;
-  if (splits < 1) splits = 1;
-  float* partial = splits > 1 ? ws.partial : nullptr;
-  dim3 grid(gm, gn, splits);
+  q.kchunk = (q.K + splits - 1) / splits;
+  q.kchunk = (q.kchunk + SB_K - 1) / SB_K * SB_K;
+  splits = (q.K + q.kchunk - 1) / q.kchunk;
+  q.partial = splits > 1 ? ws.partial : nullptr;
+  if (q.partial ? rows_of_4(q.partial, q.N, 4) : (!q.c_bf16 && rows_of_4(q.C, q.ldc, 4))) q.vec |= SIMT_VEC_C;
   if (op_bf16)
-    ::ddppo::launch_k(gemm_simt_kernel<__nv_bfloat16>, grid, 256, 0, s,
-        d.M, d.N, d.K, (const __nv_bfloat16*)d.A, d.lda, (const __nv_bfloat16*)d.B, d.ldb,
-        (float*)d.C, d.ldc, d.c_bf16, d.beta, d.bias, d.relu, kchunk, partial, d.a_t, d.b_t);
+    ::ddppo::launch_k(gemm_simt_kernel<BM, BN, TM, __nv_bfloat16>, dim3(gm, gn, splits), 256, 0, s, q);
   else
-    ::ddppo::launch_k(gemm_simt_kernel<float>, grid, 256, 0, s, d.M, d.N, d.K, (const float*)d.A, d.lda,
-                                                 (const float*)d.B, d.ldb, (float*)d.C, d.ldc,
-                                                 d.c_bf16, d.beta, d.bias, d.relu, kchunk, partial,
-                                                 d.a_t, d.b_t);
+    ::ddppo::launch_k(gemm_simt_kernel<BM, BN, TM, float>, dim3(gm, gn, splits), 256, 0, s, q);
+}
+
+static int gemm_simt(const GemmDesc& d, bool op_bf16, const GemmWorkspace& ws, cudaStream_t s) {
+  const int eb = op_bf16 ? 2 : 4;
+  SimtArgs q{};
+  q.M = d.M; q.N = d.N; q.K = d.K; q.lda = d.lda; q.ldb = d.ldb; q.ldc = d.ldc;
+  q.c_bf16 = d.c_bf16; q.relu = d.relu; q.a_t = d.a_t; q.b_t = d.b_t;
+  q.A = d.A; q.B = d.B; q.C = (float*)d.C; q.beta = d.beta; q.bias = d.bias;
+  if (rows_of_4(d.A, d.lda, eb)) q.vec |= SIMT_VEC_A;
+  if (rows_of_4(d.B, d.ldb, eb)) q.vec |= SIMT_VEC_B;
+  int splits;
+  // one tile shape leaves half its FMAs on padding for 32 channels: 128x32 and 32x128 there
+  // (9.5 us a launch; 64x64: 14.3). 128x64 saves shared reads where it still gives two CTAs
+  // an SM (19.7 us; 64x64: 20.2)
+  if (d.N <= 32) launch_simt<128, 32, 4>(q, op_bf16, ws, splits, s);
+  else if (d.M <= 32) launch_simt<32, 128, 4>(q, op_bf16, ws, splits, s);
+  else if (((d.M + 127) / 128) * (int64_t)((d.N + 63) / 64) >= 2 * ws.num_sms) launch_simt<128, 64, 8>(q, op_bf16, ws, splits, s);
+  else launch_simt<64, 64, 4>(q, op_bf16, ws, splits, s);
   DDPPO_CHECK_LAUNCH();
-  if (partial)
-    DDPPO_TRY(launch_splitk_reduce(d.M, d.N, splits, partial, (float*)d.C, d.ldc, d.c_bf16, d.beta,
-                                   d.bias, d.relu, s));
+  if (q.partial)
+    DDPPO_TRY(launch_splitk_reduce(d.M, d.N, splits, q.partial, q.C, d.ldc, d.c_bf16, d.beta, d.bias, d.relu, s));
   return DDPPO_OK;
 }
 
 int launch_splitk_reduce(int M, int N, int splits, const float* partial, float* C, int ldc,
                          int c_bf16, float beta, const float* bias, int relu, cudaStream_t s) {
   const size_t n = (size_t)M * N;
-  ::ddppo::launch_k(splitk_reduce_kernel, (unsigned)((n + 255) / 256), 256, 0, s, M, N, splits, partial, C, ldc,
-                                                                   c_bf16, beta, bias, relu);
+  // four columns a thread where that still leaves the chip (152 SMs) a block each
+  if (n >= 152 * 1024 && N % 4 == 0 && rows_of_4(partial, N, 4) && (c_bf16 || rows_of_4(C, ldc, 4)))
+    ::ddppo::launch_k(splitk_reduce_kernel<4>, (unsigned)((n / 4 + 255) / 256), 256, 0, s, M, N, splits, partial, C,
+                      ldc, c_bf16, beta, bias, relu);
+  else
+    ::ddppo::launch_k(splitk_reduce_kernel<1>, (unsigned)((n + 127) / 128), 128, 0, s, M, N, splits, partial, C,
+                      ldc, c_bf16, beta, bias, relu);
   DDPPO_CHECK_LAUNCH();
   return DDPPO_OK;
 }
