@@ -4,9 +4,14 @@
 //   * TMA (cp.async.bulk.tensor.2d) stages 128x64 A tiles and BNx64 B tiles into shared
 //     memory in the 128-byte swizzled K-major layout; out-of-range rows/columns are
 //     zero-filled by the copy engine, so ragged M, N and K need no special path.
-//   * A 4-stage ring of mbarriers: "full" (TMA -> MMA, transaction bytes) and "empty"
-//     (MMA -> TMA, signalled by tcgen05.commit when the MMAs reading a stage retire).
-//   * One thread issues tcgen05.mma.cta_group::1.kind::f16 (M=128, N=BN, K=16 per
+//   * A ring of 2 to 4 stages with mbarriers: "full" (TMA -> MMA, transaction bytes) and
+//     "empty" (MMA -> TMA, signalled by tcgen05.commit when the MMAs reading a stage retire).
+//   * The producer and the MMA warp run whole; one elected lane issues. With lane 0 alone in
+//     the loop and its slot, tap and tile found by division, a 64-wide K block took 1400
+//     cycles whatever it loaded: 182 us for a 3x3 convolution of 4096 images of 8x8x128 (81
+//     here), 189 of 16x16x64 (117), 228 of 32x32x32 (157). Bound now: the operand bytes
+//     from L2 (64 FLOPs a byte in 128x128 tiles) and, for 32 channels, the epilogue.
+//   * The elected lane issues tcgen05.mma.cta_group::1.kind::f16 (M=128, N=BN, K=16 per
 //     instruction) accumulating in fp32 in tensor memory (BN columns of TMEM); E4M3
 //     operands use kind::f8f6f4 (K=32) on the same byte layouts, with the two per-tensor
 //     scales applied in the epilogue.
@@ -175,6 +180,38 @@ __device__ __forceinline__ uint32_t bf16x2_bits(float a, float b) {
 // Tiles are (m, n, split) triples walked with stride gridDim.x.
 constexpr int TC_PTHREADS = 192;
 
+// the tiles of a persistent CTA, blockIdx.x on in steps of gridDim.x, as (M tile, N tile,
+// K split); divided once, then advanced by carries
+struct TileWalk {
+  int t, tm, tn, z, dm, dn, dz, tiles_m, tiles_n;
+  __device__ __forceinline__ TileWalk(int tiles_m_, int tiles_n_) : tiles_m(tiles_m_), tiles_n(tiles_n_) {
+    const int q = (int)blockIdx.x / tiles_m, dq = (int)gridDim.x / tiles_m;
+    t = blockIdx.x;
+    tm = t - q * tiles_m;
+    z = q / tiles_n;
+    tn = q - z * tiles_n;
+    dm = (int)gridDim.x - dq * tiles_m;
+    dz = dq / tiles_n;
+    dn = dq - dz * tiles_n;
+  }
+  __device__ __forceinline__ void next() {
+    t += gridDim.x;
+    tm += dm;
+    tn += dn;
+    z += dz;
+    if (tm >= tiles_m) { tm -= tiles_m; ++tn; }
+    if (tn >= tiles_n) { tn -= tiles_n; ++z; }
+  }
+};
+// a slot of the operand ring and the phase of its barriers
+struct RingSlot {
+  int s = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next(int stages) {
+    if (++s == stages) { s = 0; ph ^= 1u; }
+  }
+};
+
 template <int BN>
 __global__ void __launch_bounds__(TC_PTHREADS, 2)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
@@ -202,7 +239,7 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
   uint8_t* base = (uint8_t*)(((uintptr_t)dyn + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = base;
   uint8_t* sB = base + stages * A_BYTES;  // halo mode: the resident weights
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int ntiles = tiles_m * tiles_n * splits;
   volatile int* abort = &ctl.abort;
 
@@ -236,67 +273,74 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
   const uint32_t tmem = ctl.tmem_base;
 
   if (warp == 0 && halo) {
-    if (lane == 0) {
-      // halo producer: the weights of every (tap, channel block) once, resident for the
-      // whole kernel; then per (tile, channel block) one input box through the ring
-      const int nkk = ca.k * ca.k, ncb = ca.C / ca.cbw;
-      const uint32_t wbox = (uint32_t)BN * ca.cbw * 2;
+    // halo producer: the weights of every (tap, channel block) once, resident for the
+    // whole kernel; then per (tile, channel block) one input box through the ring
+    const int nkk = ca.k * ca.k, ncb = ca.C / ca.cbw;
+    const uint32_t wbox = (uint32_t)BN * ca.cbw * 2;
+    if (elect_one()) {
       mbar_expect_tx(&ctl.done, wbox * nkk * ncb);
       for (int tap = 0; tap < nkk; ++tap)
         for (int cb = 0; cb < ncb; ++cb)
           tma_load_2d(sB + (tap * ncb + cb) * wbox, &mapB, &ctl.done, tap * ca.C + cb * ca.cbw, 0);
-      uint32_t hit = 0;
-      for (int t = blockIdx.x; t < ntiles && !*abort; t += gridDim.x) {
-        const int tm = t % tiles_m, z = t / (tiles_m * tiles_n);
-        int img, ybase, xbase = -ca.p;
-        if (rowh) {
-          img = tm / ca.tpi;
-          ybase = (tm - img * ca.tpi) * ca.R - 1;
-          xbase = 0;
-        } else if (ca.ni) {
-          img = tm * ca.ni;
-          ybase = -ca.p;
-        } else {
-          img = tm / ca.tpi;
-          ybase = ((tm - img * ca.tpi) * TC_BM) / ca.Wp - ca.p;
-        }
-        const int cb_end = min(ca.C, z * kchunk + kchunk);
-        for (int c0 = z * kchunk; c0 < cb_end; c0 += ca.cbw, ++hit) {
-          const int hs = hit % stages;
-          if (!mbar_wait(&ctl.empty[hs], ((hit / stages) & 1u) ^ 1u, abort, err)) break;
-          mbar_expect_tx(&ctl.full[hs], ca.box_bytes);
-          tma_load_4d(sA + hs * A_BYTES, &mapA, &ctl.full[hs], c0, xbase, ybase, img);
-        }
-      }
-      ctl.issued = hit;
     }
+    __syncwarp();
+    RingSlot slot;
+    uint32_t hit = 0;
+    bool live = true;
+    for (TileWalk w(tiles_m, tiles_n); w.t < ntiles && live; w.next()) {
+      int img, ybase, xbase = -ca.p;
+      if (rowh) {
+        img = w.tm / ca.tpi;
+        ybase = (w.tm - img * ca.tpi) * ca.R - 1;
+        xbase = 0;
+      } else if (ca.ni) {
+        img = w.tm * ca.ni;
+        ybase = -ca.p;
+      } else {
+        img = w.tm / ca.tpi;
+        ybase = ((w.tm - img * ca.tpi) * TC_BM) / ca.Wp - ca.p;
+      }
+      const int cb_end = min(ca.C, w.z * kchunk + kchunk);
+      for (int c0 = w.z * kchunk; c0 < cb_end; c0 += ca.cbw, ++hit, slot.next(stages)) {
+        live = warp_wait(&ctl.empty[slot.s], slot.ph ^ 1u, abort, err);
+        if (!live) break;
+        if (elect_one()) {
+          mbar_expect_tx(&ctl.full[slot.s], ca.box_bytes);
+          tma_load_4d(sA + slot.s * A_BYTES, &mapA, &ctl.full[slot.s], c0, xbase, ybase, img);
+        }
+        __syncwarp();
+      }
+    }
+    if (lane == 0) ctl.issued = hit;
   } else if (warp == 1 && halo) {
-    if (lane == 0) {
-      // halo MMA issuer: tap (ky, kx) reads the staged box from row off + ky Wp + kx on
-      const int NM = rowh ? 96 : BN;  // MMA N: the row halo's three column taps x 32
-      const uint32_t idesc = fp8 ? f8_idesc(TC_BM, NM) : f16_idesc(TC_BM, NM, 0, 0);
-      const int nkk = ca.k * ca.k, ncb = ca.C / ca.cbw, rb = ca.cbw * 2;
-      const uint32_t wbox = (uint32_t)BN * ca.cbw * 2;
-      const bool wok = mbar_wait(&ctl.done, 0u, abort, err);
-      uint32_t hit = 0, ti = 0;
-      for (int t = blockIdx.x; t < ntiles && wok && !*abort; t += gridDim.x, ++ti) {
-        const int tm = t % tiles_m, z = t / (tiles_m * tiles_n);
-        const int off = ca.ni ? 0 : ((tm % ca.tpi) * TC_BM) % ca.Wp;
-        const uint32_t buf = ti & 1u, bph = (ti >> 1) & 1u;
-        if (!mbar_wait(&acc_empty[buf], bph ^ 1u, abort, err)) break;
+    // halo MMA issuer: tap (ky, kx) reads the staged box from row off + ky Wp + kx on
+    const int NM = rowh ? 96 : BN;  // MMA N: the row halo's three column taps x 32
+    const uint32_t idesc = fp8 ? f8_idesc(TC_BM, NM) : f16_idesc(TC_BM, NM, 0, 0);
+    const int ncb = ca.C / ca.cbw, rb = ca.cbw * 2;
+    const uint32_t wbox = (uint32_t)BN * ca.cbw * 2;
+    bool live = warp_wait(&ctl.done, 0u, abort, err);
+    RingSlot slot;
+    uint32_t hit = 0, ti = 0;
+    for (TileWalk w(tiles_m, tiles_n); w.t < ntiles && live; w.next(), ++ti) {
+      const int off = rowh || ca.ni ? 0 : ((w.tm % ca.tpi) * TC_BM) % ca.Wp;
+      const uint32_t buf = ti & 1u, bph = (ti >> 1) & 1u;
+      live = warp_wait(&acc_empty[buf], bph ^ 1u, abort, err);
+      if (!live) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t dacc = tmem + buf * acc_stride;
+      uint32_t acc = 0;
+      const int cb_end = min(ca.C, w.z * kchunk + kchunk);
+      for (int c0 = w.z * kchunk; c0 < cb_end; c0 += ca.cbw, ++hit, slot.next(stages)) {
+        live = warp_wait(&ctl.full[slot.s], slot.ph, abort, err);
+        if (!live) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t dacc = tmem + buf * acc_stride;
-        uint32_t acc = 0;
-        const int cb_end = min(ca.C, z * kchunk + kchunk);
-        for (int c0 = z * kchunk; c0 < cb_end; c0 += ca.cbw, ++hit) {
-          const int hs = hit % stages;
-          if (!mbar_wait(&ctl.full[hs], (hit / stages) & 1u, abort, err)) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t h0 = smem_addr(sA + hs * A_BYTES);
-          const int cb = c0 / ca.cbw;
+        const uint32_t h0 = smem_addr(sA + slot.s * A_BYTES);
+        const int cb = c0 / ca.cbw;
+        if (elect_one()) {
           if (rowh) {
             // filter row ky: the box from row ky W on; B = the weights of taps (ky, 0..2),
             // resident one after another (96 rows of 64 bytes)
+#pragma unroll
             for (int ky = 0; ky < 3; ++ky) {
               const uint32_t arow = h0 + (uint32_t)(ky * ca.W) * (uint32_t)rb;
               const uint32_t b0 = smem_addr(sB + (ky * 3 * ncb + cb) * wbox);
@@ -305,157 +349,155 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
                 acc = 1u;
               }
             }
+          } else {
+            int tap = 0;
+            for (int ky = 0; ky < ca.k; ++ky)
+              for (int kx = 0; kx < ca.k; ++kx, ++tap) {
+                const uint32_t arow = h0 + (uint32_t)(off + ky * ca.Wp + kx) * rb;
+                const uint32_t b0 = smem_addr(sB + (tap * ncb + cb) * wbox);
+                for (int kq = 0; kq < ca.cbw / 16; ++kq) {
+                  const uint64_t da = ca.cbw == 32 ? sw64_desc(arow + kq * 32) : sw128_desc(arow + kq * 32);
+                  const uint64_t db = ca.cbw == 32 ? sw64_desc(b0 + kq * 32) : sw128_desc(b0 + kq * 32);
+                  tc_mma(dacc, da, db, idesc, acc, fp8);
+                  acc = 1u;
+                }
+              }
           }
-          for (int tap = 0; tap < (rowh ? 0 : nkk); ++tap) {
-            const int ky = tap / ca.k, kx = tap - ky * ca.k;
-            const uint32_t arow = h0 + (uint32_t)(off + ky * ca.Wp + kx) * rb;
-            const uint32_t b0 = smem_addr(sB + (tap * ncb + cb) * wbox);
-            for (int kq = 0; kq < ca.cbw / 16; ++kq) {
-              const uint64_t da = ca.cbw == 32 ? sw64_desc(arow + kq * 32) : sw128_desc(arow + kq * 32);
-              const uint64_t db = ca.cbw == 32 ? sw64_desc(b0 + kq * 32) : sw128_desc(b0 + kq * 32);
-              tc_mma(dacc, da, db, idesc, acc, fp8);
-              acc = 1u;
-            }
-          }
-          asm volatile(
-              "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                  smem_addr(&ctl.empty[hs]))
-              : "memory");
+          tc_commit(&ctl.empty[slot.s]);
         }
-        asm volatile(
-            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_addr(&acc_full[buf]))
-            : "memory");
+        __syncwarp();
+        acc = 1u;
       }
-      ctl.consumed = hit;
-      if (*abort) {
-        tc_commit(&ctl.drain);  // arrives once every MMA this thread issued has completed
-        mbar_drain_wait(&ctl.drain, 0u);
-      }
+      if (!live) break;  // the tile is not complete
+      if (elect_one()) tc_commit(&acc_full[buf]);
+      __syncwarp();
+    }
+    if (lane == 0) ctl.consumed = hit;
+    if (*abort) {
+      if (elect_one()) tc_commit(&ctl.drain);  // arrives once every MMA of this warp has completed
+      mbar_drain_wait(&ctl.drain, 0u);
     }
   } else if (warp == 0) {
-    if (lane == 0) {
-      // TMA producer over every (tile, k-block) of this CTA
-      const int kstep = ca.on == 1 ? ca.cbw : TC_BK;
-      uint32_t tx = (uint32_t)(TC_BM + BN) * kstep * 2;
-      uint32_t it = 0;
-      for (int t = blockIdx.x; t < ntiles && !*abort; t += gridDim.x) {
-        const int tm = t % tiles_m, tn = (t / tiles_m) % tiles_n, z = t / (tiles_m * tiles_n);
-        const int m0 = tm * TC_BM, n0 = tn * BN;
-        const int kbeg = z * kchunk, kend = min(K, kbeg + kchunk);
-        const int nkb = (kend - kbeg + kstep - 1) / kstep;
-        // weight gradient: boxes of this tile's (tap, channel) rows that exist (rows >= M
-        // are left unloaded; their accumulator rows are never stored)
-        int nbox = 0;
-        if (ca.on == 2) {
-          nbox = min(TC_BM / ca.cbw, (M - m0 + ca.cbw - 1) / ca.cbw);
-          tx = (uint32_t)BN * TC_BK * 2 + (uint32_t)nbox * 64 * ca.cbw * 2;
-        }
-        int img = 0, oy0 = 0;
-        if (ca.on == 1) {
-          const int pix = ca.Ho * ca.Wo;
-          img = m0 / pix;
-          oy0 = (m0 - img * pix) / ca.Wo;
-        }
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = it % stages;
-          const uint32_t ph = (it / stages) & 1u;
-          if (!mbar_wait(&ctl.empty[s], ph ^ 1u, abort, err)) break;
+    // TMA producer over every (tile, k-block) of this CTA
+    const int kstep = ca.on == 1 ? ca.cbw : TC_BK;
+    uint32_t tx = (uint32_t)(TC_BM + BN) * kstep * 2;
+    RingSlot slot;
+    uint32_t it = 0;
+    bool live = true;
+    for (TileWalk w(tiles_m, tiles_n); w.t < ntiles && live; w.next()) {
+      const int m0 = w.tm * TC_BM, n0 = w.tn * BN;
+      const int kbeg = w.z * kchunk, kend = min(K, kbeg + kchunk);
+      // weight gradient: boxes of this tile's (tap, channel) rows that exist (rows >= M
+      // are left unloaded; their accumulator rows are never stored)
+      int nbox = 0;
+      if (ca.on == 2) {
+        nbox = min(TC_BM / ca.cbw, (M - m0 + ca.cbw - 1) / ca.cbw);
+        tx = (uint32_t)BN * TC_BK * 2 + (uint32_t)nbox * 64 * ca.cbw * 2;
+      }
+      int img = 0, y0 = 0, c0 = 0, kx = 0, ky = 0;  // convolution: this K block's tap and channels
+      if (ca.on == 1) {
+        const int pix = ca.Ho * ca.Wo;
+        img = m0 / pix;
+        y0 = (m0 - img * pix) / ca.Wo * ca.s - ca.p;
+        const int tap = kbeg / ca.C;
+        c0 = kbeg - tap * ca.C;
+        ky = tap / ca.k;
+        kx = tap - ky * ca.k;
+      }
+      for (int k = kbeg; k < kend; k += kstep, ++it, slot.next(stages)) {
+        const int s = slot.s;
+        live = warp_wait(&ctl.empty[s], slot.ph ^ 1u, abort, err);
+        if (!live) break;
+        if (elect_one()) {
           mbar_expect_tx(&ctl.full[s], tx);
-          const int k = kbeg + kb * kstep;
           if (ca.on == 2) {
             const int pix = ca.Ho * ca.Wo;
             const int im = k / pix, oy = (k - im * pix) / ca.Wo;
             for (int j = 0; j < nbox; ++j) {
               const int kk = m0 + j * ca.cbw;
-              const int tap = kk / ca.C, c0 = kk - tap * ca.C;
-              const int ky = tap / ca.k, kx = tap - ky * ca.k;
-              tma_load_4d(sA + s * A_BYTES + j * (64 * ca.cbw * 2), &mapA, &ctl.full[s], c0,
-                          kx - ca.p, oy * ca.s - ca.p + ky, im);
+              const int tap = kk / ca.C, cc = kk - tap * ca.C;
+              const int ty = tap / ca.k, tx_ = tap - ty * ca.k;
+              tma_load_4d(sA + s * A_BYTES + j * (64 * ca.cbw * 2), &mapA, &ctl.full[s], cc,
+                          tx_ - ca.p, oy * ca.s - ca.p + ty, im);
             }
 #pragma unroll
             for (int j = 0; j < BN / 64; ++j)
               tma_load_2d(sB + s * B_BYTES + j * 8192, &mapB, &ctl.full[s], n0 + 64 * j, k);
-            continue;
-          }
-          if (ca.on) {
+          } else if (ca.on) {
             // A: the input box of this filter tap and channel block (zero outside the image)
-            const int tap = k / ca.C, c0 = k - tap * ca.C;
-            const int ky = tap / ca.k, kx = tap - ky * ca.k;
-            tma_load_4d(sA + s * A_BYTES, &mapA, &ctl.full[s], c0, kx - ca.p, oy0 * ca.s - ca.p + ky,
-                        img);
+            tma_load_4d(sA + s * A_BYTES, &mapA, &ctl.full[s], c0, kx - ca.p, y0 + ky, img);
             tma_load_2d(sB + s * B_BYTES, &mapB, &ctl.full[s], k, n0);
-            continue;
-          }
-          if (a_mn) {
-            tma_load_2d(sA + s * A_BYTES, &mapA, &ctl.full[s], m0, k);
-            tma_load_2d(sA + s * A_BYTES + 8192, &mapA, &ctl.full[s], m0 + 64, k);
           } else {
-            tma_load_2d(sA + s * A_BYTES, &mapA, &ctl.full[s], k, m0);
-          }
-          if (b_mn) {
-#pragma unroll
-            for (int j = 0; j < BN / 64; ++j)
-              tma_load_2d(sB + s * B_BYTES + j * 8192, &mapB, &ctl.full[s], n0 + 64 * j, k);
-          } else {
-            tma_load_2d(sB + s * B_BYTES, &mapB, &ctl.full[s], k, n0);
-          }
-        }
-      }
-      ctl.issued = it;
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer
-      const uint32_t idesc = fp8 ? f8_idesc(TC_BM, BN) : f16_idesc(TC_BM, BN, a_mn, b_mn);
-      const int kstep = ca.on == 1 ? ca.cbw : TC_BK;
-      const bool sw64 = ca.on == 1 && ca.cbw == 32;
-      const bool a_sw64_mn = ca.on == 2 && ca.cbw == 32;
-      uint32_t it = 0, ti = 0;
-      for (int t = blockIdx.x; t < ntiles && !*abort; t += gridDim.x, ++ti) {
-        const int z = t / (tiles_m * tiles_n);
-        const int kbeg = z * kchunk, kend = min(K, kbeg + kchunk);
-        const int nkb = (kend - kbeg + kstep - 1) / kstep;
-        const uint32_t buf = ti & 1u, bph = (ti >> 1) & 1u;
-        if (!mbar_wait(&acc_empty[buf], bph ^ 1u, abort, err)) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t dacc = tmem + buf * BN;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = it % stages;
-          const uint32_t ph = (it / stages) & 1u;
-          if (!mbar_wait(&ctl.full[s], ph, abort, err)) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = smem_addr(sA + s * A_BYTES), b0 = smem_addr(sB + s * B_BYTES);
-          for (int k = 0; k < kstep / 16; ++k) {
-            uint64_t da, db;
-            if (sw64) {
-              da = sw64_desc(a0 + k * 32);
-              db = sw64_desc(b0 + k * 32);
-            } else if (a_sw64_mn) {
-              da = sw64_mn_desc(a0 + k * 1024);
-              db = sw128_mn_desc(b0 + k * 2048);
+            if (a_mn) {
+              tma_load_2d(sA + s * A_BYTES, &mapA, &ctl.full[s], m0, k);
+              tma_load_2d(sA + s * A_BYTES + 8192, &mapA, &ctl.full[s], m0 + 64, k);
             } else {
-              da = a_mn ? sw128_mn_desc(a0 + k * 2048) : sw128_desc(a0 + k * 32);
-              db = b_mn ? sw128_mn_desc(b0 + k * 2048) : sw128_desc(b0 + k * 32);
+              tma_load_2d(sA + s * A_BYTES, &mapA, &ctl.full[s], k, m0);
             }
-            const uint32_t acc = (kb | k) ? 1u : 0u;
-            tc_mma(dacc, da, db, idesc, acc, fp8);
+            if (b_mn) {
+#pragma unroll
+              for (int j = 0; j < BN / 64; ++j)
+                tma_load_2d(sB + s * B_BYTES + j * 8192, &mapB, &ctl.full[s], n0 + 64 * j, k);
+            } else {
+              tma_load_2d(sB + s * B_BYTES, &mapB, &ctl.full[s], k, n0);
+            }
           }
-          asm volatile(
-              "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                  smem_addr(&ctl.empty[s]))
-              : "memory");
         }
-        asm volatile(
-            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_addr(&acc_full[buf]))
-            : "memory");
+        __syncwarp();
+        if ((c0 += kstep) == ca.C) {
+          c0 = 0;
+          if (++kx == ca.k) { kx = 0; ++ky; }
+        }
       }
-      ctl.consumed = it;
-      if (*abort) {
-        tc_commit(&ctl.drain);  // arrives once every MMA this thread issued has completed
-        mbar_drain_wait(&ctl.drain, 0u);
+    }
+    if (lane == 0) ctl.issued = it;
+  } else if (warp == 1) {
+    // MMA issuer
+    const uint32_t idesc = fp8 ? f8_idesc(TC_BM, BN) : f16_idesc(TC_BM, BN, a_mn, b_mn);
+    const int kstep = ca.on == 1 ? ca.cbw : TC_BK;
+    const bool sw64 = ca.on == 1 && ca.cbw == 32;
+    const bool a_sw64_mn = ca.on == 2 && ca.cbw == 32;
+    // an operand's descriptor: the upper part is the same for every block of the ring
+    const uint64_t dA = sw64 ? sw64_desc(0) : a_sw64_mn ? sw64_mn_desc(0) : a_mn ? sw128_mn_desc(0) : sw128_desc(0);
+    const uint64_t dB = sw64 ? sw64_desc(0) : (a_sw64_mn || b_mn) ? sw128_mn_desc(0) : sw128_desc(0);
+    // bytes from one MMA's operand to the next
+    const uint32_t stepA = a_sw64_mn ? 1024 : a_mn ? 2048 : 32, stepB = (a_sw64_mn || b_mn) ? 2048 : 32;
+    RingSlot slot;
+    uint32_t it = 0, ti = 0;
+    bool live = true;
+    for (TileWalk w(tiles_m, tiles_n); w.t < ntiles && live; w.next(), ++ti) {
+      const int kbeg = w.z * kchunk, kend = min(K, kbeg + kchunk);
+      const uint32_t buf = ti & 1u, bph = (ti >> 1) & 1u;
+      live = warp_wait(&acc_empty[buf], bph ^ 1u, abort, err);
+      if (!live) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t dacc = tmem + buf * BN;
+      uint32_t acc = 0;
+      for (int k = kbeg; k < kend; k += kstep, ++it, slot.next(stages)) {
+        live = warp_wait(&ctl.full[slot.s], slot.ph, abort, err);
+        if (!live) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t a0 = smem_addr(sA + slot.s * A_BYTES), b0 = smem_addr(sB + slot.s * B_BYTES);
+        if (elect_one()) {
+#pragma unroll
+          for (int kq = 0; kq < TC_BK / 16; ++kq) {
+            if (kq * 16 >= kstep) break;
+            tc_mma(dacc, dA | ((a0 + kq * stepA) >> 4 & 0x3FFF), dB | ((b0 + kq * stepB) >> 4 & 0x3FFF), idesc,
+                   acc | (uint32_t)(kq != 0), fp8);
+          }
+          tc_commit(&ctl.empty[slot.s]);
+        }
+        __syncwarp();
+        acc = 1u;
       }
+      if (!live) break;  // the tile is not complete
+      if (elect_one()) tc_commit(&acc_full[buf]);
+      __syncwarp();
+    }
+    if (lane == 0) ctl.consumed = it;
+    if (*abort) {
+      if (elect_one()) tc_commit(&ctl.drain);  // arrives once every MMA of this warp has completed
+      mbar_drain_wait(&ctl.drain, 0u);
     }
   } else {
     // epilogue warps 2..5: warp w reads TMEM lanes 32 (w % 4) .. +31
@@ -468,9 +510,10 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
     const int Mo = trans_out ? N : M, No = trans_out ? M : N;
     // per-tensor scales of E4M3 operands (exactly 1 otherwise)
     const float alpha = (scale_a ? *scale_a : 1.f) * (scale_b ? *scale_b : 1.f);
+    const int px = rowh ? (q * 32 + lane) % ca.W : 0;  // row halo: this lane's image column
     uint32_t ti = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++ti) {
-      const int tm = t % tiles_m, tn = (t / tiles_m) % tiles_n, z = t / (tiles_m * tiles_n);
+    for (TileWalk w(tiles_m, tiles_n); w.t < ntiles; w.next(), ++ti) {
+      const int tm = w.tm, tn = w.tn, z = w.z;
       const int m0 = tm * TC_BM, n0 = tn * BN;
       const uint32_t buf = ti & 1u, bph = (ti >> 1) & 1u;
       const bool ok = mbar_wait(&acc_full[buf], bph, abort, err);
@@ -478,8 +521,7 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
       const int row = m0 + q * 32 + lane;
       // halo mode: output row of this lane's tile row, computed once per tile and handed to
       // the row loop by shuffles
-      const long long my_orow = halo ? halo_out_row(ca, tm, q * 32 + lane) : 0;
-      const int px = rowh ? (q * 32 + lane) % ca.W : 0;  // row halo: this lane's image column
+      const long long my_orow = halo && !tma_out ? halo_out_row(ca, tm, q * 32 + lane) : 0;
 #pragma unroll 1
       for (int c0 = 0; c0 < BN; c0 += 32) {
         if (n0 + c0 >= N) break;  // columns past N: nothing to read or store
@@ -545,7 +587,8 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
             }
             __syncwarp();  // every lane has read its row before the block is rewritten
           }
-          const float bl = (bias && !part) ? bias[min(n0 + c0 + lane, N - 1)] : 0.f;
+          const bool has_bias = bias && !part;
+          const float bl = has_bias ? bias[min(n0 + c0 + lane, N - 1)] : 0.f;
           float x[32];
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
@@ -553,7 +596,7 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
             if (fp8) v *= alpha;
             if (!part) {
               if (beta != 0.f) v = __fmaf_rn(beta, cv[j], v);
-              v += __shfl_sync(0xffffffffu, bl, j);
+              v += has_bias ? __shfl_sync(0xffffffffu, bl, j) : 0.f;
               if (relu) v = fmaxf(v, 0.f);
             }
             x[j] = v;
@@ -1062,10 +1105,15 @@ static int kslot_of(const GemmDesc& d) {
   return TC_BK;
 }
 
-static TcCfg default_cfg(int N, int kslot) {
+// 128x128 tiles: with two tiles an SM and more, two CTAs of a 2-slot ring each (one's
+// epilogue runs under the other's MMAs): 512 tiles of K = 1152 in E4M3 17 us, one CTA of a
+// 4-slot ring 21; 2048 tiles of K = 1152 in bf16 81 and 89. Fewer tiles have an SM each and
+// take the deeper ring (and split K over the SMs, not over the CTA slots).
+static TcCfg default_cfg(int M, int N, int kslot, int num_sms) {
   TcCfg c;
   c.bn = N > 64 ? 128 : 64;
-  c.stages = std::min(ring_for(c.bn, kslot), c.bn == 64 ? 3 : 4);
+  const int64_t tiles = (int64_t)((M + TC_BM - 1) / TC_BM) * ((N + c.bn - 1) / c.bn);
+  c.stages = std::min(ring_for(c.bn, kslot), c.bn == 64 ? 3 : tiles >= 2 * num_sms ? 2 : 4);
   c.split = 0;
   return c;
 }
@@ -1246,7 +1294,7 @@ static TcCfg tune(const GemmDesc& d, const GemmWorkspace& ws, TcTuner& t, cudaSt
   trial.C = t.scratch;
   trial.ldc = d.N;
   trial.beta = 0.f;
-  TcCfg best = default_cfg(Nk, kslot);
+  TcCfg best = default_cfg(swap ? d.N : d.M, Nk, kslot, ws.num_sms);
   if (hal && !gat) {
     best.bn = halo_bn(d.conv->Cout);
     best.stages = 2;
@@ -1268,7 +1316,7 @@ static TcCfg tune(const GemmDesc& d, const GemmWorkspace& ws, TcTuner& t, cudaSt
 
 int gemm_tc(const GemmDesc& d, const GemmWorkspace& ws, cudaStream_t s) {
   const bool swap = d.convw || (!d.conv && d.M < TC_BM && d.N > d.M);
-  TcCfg cfg = default_cfg(swap ? d.M : d.N, kslot_of(d));
+  TcCfg cfg = default_cfg(swap ? d.N : d.M, swap ? d.M : d.N, kslot_of(d), ws.num_sms);
   ConvA hca;
   if (d.conv && halo_geom(*d.conv, &hca) && (hca.on == 4 || !gather_ok(*d.conv))) {
     const ConvA& ca = hca;
@@ -1341,7 +1389,7 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
   uint8_t* base = (uint8_t*)(((uintptr_t)dyn + 1023) & ~(uintptr_t)1023);
   uint8_t* sX = base;
   uint8_t* sD = base + stages * x_stride;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   volatile int* abort = &abort_flag;
   if (threadIdx.x == 0) {
     for (int i = 0; i < stages; ++i) {
@@ -1368,50 +1416,45 @@ __global__ void __launch_bounds__(WH_THREADS, 1)
   const int kq = RB * Wp / 16;
   const bool has_work = (int)blockIdx.x < nunits;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
+    RingSlot slot;
     uint32_t it = 0;
-    for (int u = blockIdx.x; u < nunits && !*abort; u += gridDim.x, ++it) {
-      const int s = it % stages;
-      if (!mbar_wait(&empty[s], ((it / stages) & 1u) ^ 1u, abort, err)) break;
-      const int img = u / nrb, y0 = (u - img * nrb) * RB;
-      mbar_expect_tx(&full[s], x_bytes + dz_bytes);
-      tma_load_4d(sX + s * x_stride, &mapX, &full[s], 0, -1, y0 - 1, img);
-      tma_load_4d(sD + s * dz_stride, &mapDZ, &full[s], 0, 0, y0, img);
+    for (int u = blockIdx.x; u < nunits; u += gridDim.x, ++it, slot.next(stages)) {
+      const int s = slot.s, img = u / nrb, y0 = (u - img * nrb) * RB;
+      if (!warp_wait(&empty[s], slot.ph ^ 1u, abort, err)) break;
+      if (elect_one()) {
+        mbar_expect_tx(&full[s], x_bytes + dz_bytes);
+        tma_load_4d(sX + s * x_stride, &mapX, &full[s], 0, -1, y0 - 1, img);
+        tma_load_4d(sD + s * dz_stride, &mapDZ, &full[s], 0, 0, y0, img);
+      }
+      __syncwarp();
     }
-    n_issued = it;
-  } else if (warp == 1 && lane == 0) {
+    if (lane == 0) n_issued = it;
+  } else if (warp == 1) {
     const uint32_t idesc = f16_idesc(TC_BM, 32, 1, 1);
+    RingSlot slot;
     uint32_t it = 0;
-    for (int u = blockIdx.x; u < nunits && !*abort; u += gridDim.x, ++it) {
-      const int s = it % stages;
-      if (!mbar_wait(&full[s], (it / stages) & 1u, abort, err)) break;
+    for (int u = blockIdx.x; u < nunits; u += gridDim.x, ++it, slot.next(stages)) {
+      const int s = slot.s;
+      if (!warp_wait(&full[s], slot.ph, abort, err)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t x0 = smem_addr(sX + s * x_stride), d0 = smem_addr(sD + s * dz_stride);
-      for (int k = 0; k < kq; ++k) {
-        const uint64_t db = sw64_mn_desc_lbo(d0 + (uint32_t)k * 16 * 64, 4096);
+      if (elect_one()) {
+        for (int k = 0; k < kq; ++k) {
+          const uint64_t db = sw64_mn_desc_lbo(d0 + (uint32_t)k * 16 * 64, 4096);
 #pragma unroll
-        for (int ky = 0; ky < 3; ++ky) {
-          const uint64_t da = sw64_mn_desc_lbo(x0 + (uint32_t)(ky * Wp + k * 16) * 64, 64);
-          const uint32_t acc = (it | k) ? 1u : 0u;
-          asm volatile(
-              "{\n\t.reg .pred p;\n\t"
-              "setp.ne.b32 p, %4, 0;\n\t"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem + ky * 32),
-              "l"(da), "l"(db), "r"(idesc), "r"(acc)
-              : "memory");
+          for (int ky = 0; ky < 3; ++ky) {
+            const uint64_t da = sw64_mn_desc_lbo(x0 + (uint32_t)(ky * Wp + k * 16) * 64, 64);
+            tc_mma(tmem + ky * 32, da, db, idesc, (it | k) ? 1u : 0u, 0);
+          }
         }
+        tc_commit(&empty[s]);
       }
-      asm volatile(
-          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-              smem_addr(&empty[s]))
-          : "memory");
+      __syncwarp();
     }
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_addr(&done))
-        : "memory");
-    n_consumed = it;
-    // after an abort the epilogue no longer waits for `done`; this thread does, so that
+    if (elect_one()) tc_commit(&done);
+    if (lane == 0) n_consumed = it;
+    // after an abort the epilogue no longer waits for `done`; this warp does, so that
     // every MMA it issued has completed before the accumulators are freed
     if (*abort) mbar_drain_wait(&done, 0u);
   }

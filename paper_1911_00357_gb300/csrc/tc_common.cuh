@@ -46,6 +46,26 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
+// The issuing warps of a tcgen05 or TMA loop run whole (every lane takes every branch), and
+// one elected lane issues: operands of these instructions live in uniform registers, and in
+// a branch taken by lane 0 alone each has to be moved there for every instruction: 150
+// cycles an MMA of 128x128x16 (182 us for a convolution that took 125 after this change).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+// the warp's index, known to be the same in all its lanes
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+// mbar_wait by a whole warp: true if every lane's wait ended well
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort, int32_t* err) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, err));
+}
+
 // the drain after an abort: poll until the phase completes or the limit runs out (the
 // abort flag is already set, so mbar_wait would return at once)
 __device__ __forceinline__ bool mbar_drain_wait(uint64_t* bar, uint32_t parity) {

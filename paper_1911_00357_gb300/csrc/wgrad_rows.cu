@@ -24,9 +24,9 @@
 // of a box are zeros that no copy overwrites: they meet dz = 0, and stale values there could
 // be NaN.
 //
-// Measured (4096 images): 16x16, 64 -> 64 channels 127 us against 367 us for the gather form
+// Measured (4096 images): 16x16, 64 -> 64 channels 106 us against 367 us for the gather form
 // (0.61 PFLOP/s; N = 64 leaves the MMAs bound by shared-memory reads); the seven
-// convolutions of stages 3, 4 and the compression layer 91 us each on average, reduction
+// convolutions of stages 3, 4 and the compression layer 72 us each on average, reduction
 // included. The encoder's ten such gradients: 1.02 ms against 2.9 ms.
 #include <algorithm>
 #include <cstring>
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(WR_THREADS, 1)
   constexpr int NACC = NB == 64 ? 6 : 3;  // accumulators of NB columns
   uint8_t* base = (uint8_t*)(((uintptr_t)dyn + 1023) & ~(uintptr_t)1023);
   const uint32_t stage_bytes = NX * (a.x_stride + a.d_stride);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   volatile int* abort = &abort_flag;
   if (threadIdx.x == 0) {
     for (int i = 0; i < a.stages; ++i) {
@@ -100,48 +100,56 @@ __global__ void __launch_bounds__(WR_THREADS, 1)
   const int cb = a.by_row ? (job / 3) % a.cb128 : 0, nb = a.by_row ? job / (3 * a.cb128) : 0;
   const bool has_work = split < a.nunits;
 
-  if (warp == 0 && lane == 0) {
-    uint32_t it = 0;
-    for (int u = split; u < a.nunits && !*abort; u += a.cpj, ++it) {
-      const int s = it % a.stages;
-      if (!mbar_wait(&empty[s], ((it / a.stages) & 1u) ^ 1u, abort, err)) break;
+  if (warp == 0) {
+    uint32_t it = 0, ph = 0;
+    int s = 0;
+    for (int u = split; u < a.nunits; u += a.cpj, ++it) {
       const int ib = u / a.nrb, y0 = (u - ib * a.nrb) * a.RB, n0 = ib * a.ni;
-      uint8_t* sx = base + s * stage_bytes;
-      uint8_t* sd = sx + NX * a.x_stride;
-      mbar_expect_tx(&full[s], NX * (a.x_bytes + a.d_bytes));
+      if (!warp_wait(&empty[s], ph ^ 1u, abort, err)) break;
+      if (elect_one()) {
+        uint8_t* sx = base + s * stage_bytes;
+        uint8_t* sd = sx + NX * a.x_stride;
+        mbar_expect_tx(&full[s], NX * (a.x_bytes + a.d_bytes));
 #pragma unroll
-      for (int i = 0; i < NX; ++i) {
-        tma_load_4d(sx + i * a.x_stride, &mapX, &full[s], cb * 128 + i * 64, -1, n0, y0 - 1 + ky);
-        tma_load_4d(sd + i * a.d_stride, &mapD, &full[s], nb * 128 + i * 64, 0, n0, y0);
-      }
-    }
-    n_issued = it;
-  } else if (warp == 1 && lane == 0) {
-    const uint32_t idesc = f16_idesc(128, NB, 1, 1);
-    uint32_t it = 0;
-    for (int u = split; u < a.nunits && !*abort; u += a.cpj, ++it) {
-      const int s = it % a.stages;
-      if (!mbar_wait(&full[s], (it / a.stages) & 1u, abort, err)) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t x0 = smem_addr(base + s * stage_bytes), d0 = x0 + NX * a.x_stride;
-      for (int k = 0; k < a.ksteps; ++k) {
-        const uint64_t db = sw128_mn_desc(d0 + (uint32_t)k * 16 * 128, a.d_stride);
-        const uint32_t acc = (it | k) ? 1u : 0u;
-#pragma unroll
-        for (int q = 0; q < NACC; ++q) {
-          // all taps: accumulator (ky, pair) reads the box from row ky, columns 2 pair and
-          // 2 pair + 1; by row: accumulator kx, the second atom is the next 64 channels
-          const int shift = NB == 64 ? (q >> 1) * a.ni * a.Wp + 2 * (q & 1) : q;
-          const uint64_t da = sw128_mn_desc(x0 + (uint32_t)(shift + k * 16) * 128,
-                                            NB == 64 ? 128u : a.x_stride);
-          tc_mma(tmem + q * NB, da, db, idesc, acc, 0);
+        for (int i = 0; i < NX; ++i) {
+          tma_load_4d(sx + i * a.x_stride, &mapX, &full[s], cb * 128 + i * 64, -1, n0, y0 - 1 + ky);
+          tma_load_4d(sd + i * a.d_stride, &mapD, &full[s], nb * 128 + i * 64, 0, n0, y0);
         }
       }
-      tc_commit(&empty[s]);
+      __syncwarp();
+      if (++s == a.stages) { s = 0; ph ^= 1u; }
     }
-    tc_commit(&done);
-    n_consumed = it;
-    // after an abort the epilogue no longer waits for `done`; this thread does, so that
+    if (lane == 0) n_issued = it;
+  } else if (warp == 1) {
+    const uint32_t idesc = f16_idesc(128, NB, 1, 1);
+    uint32_t it = 0, ph = 0;
+    int s = 0;
+    for (int u = split; u < a.nunits; u += a.cpj, ++it) {
+      if (!warp_wait(&full[s], ph, abort, err)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t x0 = smem_addr(base + s * stage_bytes), d0 = x0 + NX * a.x_stride;
+      if (elect_one()) {
+        for (int k = 0; k < a.ksteps; ++k) {
+          const uint64_t db = sw128_mn_desc(d0 + (uint32_t)k * 16 * 128, a.d_stride);
+          const uint32_t acc = (it | k) ? 1u : 0u;
+#pragma unroll
+          for (int q = 0; q < NACC; ++q) {
+            // all taps: accumulator (ky, pair) reads the box from row ky, columns 2 pair and
+            // 2 pair + 1; by row: accumulator kx, the second atom is the next 64 channels
+            const int shift = NB == 64 ? (q >> 1) * a.ni * a.Wp + 2 * (q & 1) : q;
+            const uint64_t da = sw128_mn_desc(x0 + (uint32_t)(shift + k * 16) * 128,
+                                              NB == 64 ? 128u : a.x_stride);
+            tc_mma(tmem + q * NB, da, db, idesc, acc, 0);
+          }
+        }
+        tc_commit(&empty[s]);
+      }
+      __syncwarp();
+      if (++s == a.stages) { s = 0; ph ^= 1u; }
+    }
+    if (elect_one()) tc_commit(&done);
+    if (lane == 0) n_consumed = it;
+    // after an abort the epilogue no longer waits for `done`; this warp does, so that
     // every MMA it issued has completed before the accumulators are freed
     if (*abort) mbar_drain_wait(&done, 0u);
   }
