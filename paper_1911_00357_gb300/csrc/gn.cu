@@ -1276,19 +1276,23 @@ int launch_gn_bwd(const GNBack& b, int N, int HW, int C, const GnScratch& w, int
 }
 
 // ---- GroupNorm apply + ReLU + 3x3 / stride-2 / pad-1 max pool (4 channels per thread) ----
-__global__ void __launch_bounds__(kThreads) gn_relu_maxpool_kernel(GNApply a, int H, int W, int C,
+// A thread walks down a column of windows: of a window's three input rows the first is the
+// last of the window above, kept normalised, so it loads six pixels and not nine, all in
+// flight at once. Each window compares in (ky, kx) order. Bound: HBM -- z once, the pooled
+// outputs once (3.0 GB for 4096 images of 64x64x32). Nine loads a window one after another
+// took 959 us there; this form 595 (5.0 TB/s).
+__global__ void __launch_bounds__(kThreads) gn_relu_maxpool_kernel(GNApply a, int H, int W, int C, int rows,
                                                                    float* __restrict__ pool,
                                                                    __nv_bfloat16* __restrict__ pool_bf,
                                                                    uint8_t* __restrict__ arg) {
   DDPPO_PDL_ENTRY();
   const int Hq = (H - 1) / 2 + 1, Wq = (W - 1) / 2 + 1, C4 = C / 4, G = C / 2;
-  const int n = blockIdx.y, per = Hq * Wq * C4;
+  const int n = blockIdx.y, p0 = blockIdx.x * rows, p1 = min(Hq, p0 + rows);
   const float* zi = a.z + (size_t)n * H * W * C;
   const float f8s = a.out_f8 ? *a.f8_scale : 1.f;
   float f8m = 0.f;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < per; i += gridDim.x * blockDim.x) {
-    const int c4 = i % C4, pix = i / C4, c0 = c4 * 4;
-    const int ox = pix % Wq, oy = pix / Wq;
+  for (int i = threadIdx.x; i < Wq * C4; i += kThreads) {
+    const int q = i / C4, c0 = (i - q * C4) * 4;
     float gm[4], bt[4], mu[4], rs[4];
     ldv<4>(a.gamma + c0, gm);
     ldv<4>(a.beta + c0, bt);
@@ -1297,32 +1301,55 @@ __global__ void __launch_bounds__(kThreads) gn_relu_maxpool_kernel(GNApply a, in
       mu[v] = a.mean[(size_t)n * G + (c0 + v) / 2];
       rs[v] = a.rstd[(size_t)n * G + (c0 + v) / 2];
     }
-    float best[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-    int bi[4] = {0, 0, 0, 0};
-    for (int ky = 0; ky < 3; ++ky) {
-      const int iy = oy * 2 - 1 + ky;
-      if (iy < 0 || iy >= H) continue;
-      for (int kx = 0; kx < 3; ++kx) {
-        const int ix = ox * 2 - 1 + kx;
-        if (ix < 0 || ix >= W) continue;
-        float x[4];
-        ldv<4>(zi + ((size_t)iy * W + ix) * C + c0, x);
+    const int x0 = 2 * q - 1;
+    const bool in[3] = {x0 >= 0, true, x0 + 2 < W};
+    // normalised rows of the column's three pixels; pixels outside count as -infinity
+    const auto load = [&](int iy, float (&x)[3][4]) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if (in[k] && iy >= 0 && iy < H) ldv<4>(zi + ((size_t)iy * W + x0 + k) * C + c0, x[k]);
+    };
+    const auto norm = [&](int iy, float (&x)[3][4]) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+          x[k][v] = in[k] && iy >= 0 && iy < H ? fmaxf(normalised(x[k][v], mu[v], rs[v], gm[v], bt[v]), 0.f)
+                                               : -INFINITY;
+    };
+    float top[3][4];
+    load(2 * p0 - 1, top);
+    norm(2 * p0 - 1, top);
+#pragma unroll 1
+    for (int p = p0; p < p1; ++p) {
+      float mid[3][4], bot[3][4];
+      load(2 * p, mid);
+      load(2 * p + 1, bot);
+      norm(2 * p, mid);
+      norm(2 * p + 1, bot);
+      float best[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+      int bi[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int k = 0; k < 9; ++k)
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-          const float y = fmaxf(normalised(x[v], mu[v], rs[v], gm[v], bt[v]), 0.f);
-          if (y > best[v]) { best[v] = y; bi[v] = ky * 3 + kx; }
+          const float y = k < 3 ? top[k % 3][v] : k < 6 ? mid[k % 3][v] : bot[k % 3][v];
+          if (y > best[v]) { best[v] = y; bi[v] = k; }
         }
-      }
-    }
-    const size_t o = (size_t)n * per * 4 + (size_t)i * 4;
-    stv<4>(pool + o, best);
-    if (pool_bf) stv_bf<4>(pool_bf + o, best);
-    if (a.out_f8) {
-      stv_e4m3<4>(a.out_f8 + o, best, f8s);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) f8m = fmaxf(f8m, best[v]);
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) top[k][v] = bot[k][v];
+      const size_t o = (((size_t)n * Hq + p) * Wq + q) * C + c0;
+      stv<4>(pool + o, best);
+      if (pool_bf) stv_bf<4>(pool_bf + o, best);
+      if (a.out_f8) {
+        stv_e4m3<4>(a.out_f8 + o, best, f8s);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) f8m = fmaxf(f8m, best[v]);
+      }
+      *reinterpret_cast<uchar4*>(arg + o) = make_uchar4(bi[0], bi[1], bi[2], bi[3]);
     }
-    *reinterpret_cast<uchar4*>(arg + o) = make_uchar4(bi[0], bi[1], bi[2], bi[3]);
   }
   if (a.out_f8) block_amax(f8m, a.f8_amax);
 }
@@ -1335,11 +1362,10 @@ int launch_gn_relu_maxpool(const GNApply& a, int N, int H, int W, int C, float* 
     set_error("gn_relu_maxpool: unsupported shape");
     return DDPPO_E_CONFIG;
   }
-  const long per = (long)Hq * Wq * (C / 4);
-  const dim3 gb((unsigned)std::max<long>(1, std::min<long>((per + kThreads - 1) / kThreads,
-                                                           (8l * num_sms_cached() + N - 1) / N)),
-                N);
-  ::ddppo::launch_k(gn_relu_maxpool_kernel, gb, kThreads, 0, s, a, H, W, C, pool, pool_bf, arg);
+  // few images: their rows over several blocks (each normalises the row above its first again)
+  const int rows = std::max(1, (int)std::min<long>(Hq, (long)N * Hq / (8l * num_sms_cached())));
+  ::ddppo::launch_k(gn_relu_maxpool_kernel, dim3((Hq + rows - 1) / rows, N), kThreads, 0, s, a, H, W, C, rows, pool,
+                    pool_bf, arg);
   DDPPO_CHECK_LAUNCH();
   return DDPPO_OK;
 }
