@@ -339,6 +339,13 @@ static bool conv_c1_ok(const GemmDesc& d) {
          d.ldb >= d.conv->k * d.conv->k;
 }
 
+// the stem's weight gradient: N is the padded tap count of the GEMM-layout gradient
+static bool wgrad_stem_ok(const GemmDesc& d, bool op_bf16, const GemmWorkspace& ws) {
+  return d.convw && op_bf16 && !d.conv && d.a_t && d.lda == d.M && !d.c_bf16 && !d.bias && !d.relu && !d.fp8 &&
+         d.M == d.convw->Cout && d.N >= 49 && d.N <= 64 && d.ldc == d.N &&
+         d.K == d.convw->N * d.convw->Ho * d.convw->Wo && conv_wgrad_stem_ok(*d.convw, d.B, d.A, ws);
+}
+
 int gemm(const GemmDesc& d, bool op_bf16, const GemmWorkspace& ws, cudaStream_t s,
          KernelTimer* timer) {
   if (d.M <= 0 || d.N <= 0) return DDPPO_OK;
@@ -358,7 +365,8 @@ int gemm(const GemmDesc& d, bool op_bf16, const GemmWorkspace& ws, cudaStream_t 
     set_error("gemm: implicit convolution not supported for this shape");
     return DDPPO_E_CONFIG;
   }
-  if (d.convw && !(op_bf16 && !d.conv && d.a_t && d.lda == d.M && d.lda % 8 == 0 && !d.c_bf16 && !d.bias && !d.relu &&
+  const bool stem_w = wgrad_stem_ok(d, op_bf16, ws);
+  if (d.convw && !stem_w && !(op_bf16 && !d.conv && d.a_t && d.lda == d.M && d.lda % 8 == 0 && !d.c_bf16 && !d.bias && !d.relu &&
                    d.N == d.convw->k * d.convw->k * d.convw->C &&
                    d.K == d.convw->N * d.convw->Ho * d.convw->Wo &&
                    (conv_wgrad_halo_ok(*d.convw, d.B, d.A) ||
@@ -379,6 +387,18 @@ int gemm(const GemmDesc& d, bool op_bf16, const GemmWorkspace& ws, cudaStream_t 
   int rc;
   if (d.fp8) {
     rc = gemm_fp8(d, ws, s);
+    if (ws.tc && ws.tc->on) {
+      ws.tc->launches += 1;
+      ws.tc->flops += 2.0 * d.M * d.N * d.K;
+    }
+  } else if (stem_w) {
+    rc = conv_wgrad_stem(*d.convw, d.B, d.A, (float*)d.C, d.ldc, d.beta, ws, s);
+    if (ws.tc && ws.tc->on) {
+      ws.tc->launches += 1;
+      ws.tc->flops += 2.0 * d.M * d.N * d.K;
+    }
+  } else if (op_bf16 && conv_c1_ok(d) && conv_stem_ok(*d.conv, d.A) && !((uintptr_t)d.C & 15)) {
+    rc = conv_stem(*d.conv, d.A, d.B, d.ldb, (float*)d.C, d.beta, ws, s);
     if (ws.tc && ws.tc->on) {
       ws.tc->launches += 1;
       ws.tc->flops += 2.0 * d.M * d.N * d.K;

@@ -656,6 +656,12 @@ static int conv_fwd(Net& n, ConvL& c, const void* in, bool in_bf16, int N, float
     d.A = in_bf; d.lda = d.K;
     return G(n, d, s);
   }
+  const void* x_bf = in_bf ? (const void*)in_bf : (in_bf16 ? in : nullptr);
+  if (n.bf && x_bf && !bias_relu && conv_stem_ok(cs, x_bf)) {
+    d.conv = &cs;  // the stem builds its patches in shared memory
+    d.A = x_bf; d.lda = c.Kp;
+    return G(n, d, s);
+  }
   const ConvGeom g = geom(c, N);
   if (n.bf && in_bf) DDPPO_TRY(launch_im2col(g, in_bf, true, n.col, n.bf, false, s));
   else DDPPO_TRY(launch_im2col(g, in, in_bf16, n.col, n.bf, false, s));
@@ -680,6 +686,9 @@ static int conv_bwd(Net& n, ConvL& c, const void* in, bool in_bf16, int N, const
   if (n.bf && x_bf && c.Kp == c.k * c.k * c.cin && c.cout % 8 == 0 &&
       (conv_wgrad_halo_ok(cs, x_bf, dzop) || gemm_convw_supported(cs, x_bf, dzop))) {
     w.convw = &cs;  // the GEMM gathers the shifted input rows itself
+    w.B = x_bf;
+  } else if (n.bf && x_bf && conv_wgrad_stem_ok(cs, x_bf, dzop, n.gws)) {
+    w.convw = &cs;  // the stem: taps padded to c.Kp
     w.B = x_bf;
   } else {
     if (in_bf) DDPPO_TRY(launch_im2col(g, in_bf, true, n.col, n.bf, false, s));

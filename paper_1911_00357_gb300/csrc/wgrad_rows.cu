@@ -25,9 +25,9 @@
 // be NaN.
 //
 // Measured (4096 images): 16x16, 64 -> 64 channels 106 us against 367 us for the gather form
-// (0.61 PFLOP/s; N = 64 leaves the MMAs bound by shared-memory reads); the seven
+// (0.73 PFLOP/s; N = 64 leaves the MMAs bound by shared-memory reads); the seven
 // convolutions of stages 3, 4 and the compression layer 72 us each on average, reduction
-// included. The encoder's ten such gradients: 1.02 ms against 2.9 ms.
+// included. The encoder's ten such gradients: 0.80 ms against 2.9 ms.
 #include <algorithm>
 #include <cstring>
 
