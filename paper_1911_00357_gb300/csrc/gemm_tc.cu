@@ -381,6 +381,9 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
     // TMA producer over every (tile, k-block) of this CTA
     const int kstep = ca.on == 1 ? ca.cbw : TC_BK;
     uint32_t tx = (uint32_t)(TC_BM + BN) * kstep * 2;
+    // weight gradient: a 64-pixel K block is so many rows of an image, or so many images
+    const int wg_imgs = ca.on == 2 && ca.Ho * ca.Wo <= TC_BK ? TC_BK / (ca.Ho * ca.Wo) : 0;
+    const int wg_rows = ca.on == 2 && !wg_imgs ? TC_BK / ca.Wo : 0;
     RingSlot slot;
     uint32_t it = 0;
     bool live = true;
@@ -393,6 +396,20 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
       if (ca.on == 2) {
         nbox = min(TC_BM / ca.cbw, (M - m0 + ca.cbw - 1) / ca.cbw);
         tx = (uint32_t)BN * TC_BK * 2 + (uint32_t)nbox * 64 * ca.cbw * 2;
+      }
+      // ... their taps and channels, and the image and output row of the first K block
+      int bc[4] = {}, bx[4] = {}, by[4] = {}, im = 0, oy = 0;
+      if (ca.on == 2) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int kk = m0 + j * ca.cbw, tap = kk / ca.C, fy = tap / ca.k;
+          bc[j] = kk - tap * ca.C;
+          bx[j] = tap - fy * ca.k - ca.p;
+          by[j] = fy - ca.p;
+        }
+        const int pix = ca.Ho * ca.Wo;
+        im = kbeg / pix;
+        oy = (kbeg - im * pix) / ca.Wo;
       }
       int img = 0, y0 = 0, c0 = 0, kx = 0, ky = 0;  // convolution: this K block's tap and channels
       if (ca.on == 1) {
@@ -411,15 +428,11 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
         if (elect_one()) {
           mbar_expect_tx(&ctl.full[s], tx);
           if (ca.on == 2) {
-            const int pix = ca.Ho * ca.Wo;
-            const int im = k / pix, oy = (k - im * pix) / ca.Wo;
-            for (int j = 0; j < nbox; ++j) {
-              const int kk = m0 + j * ca.cbw;
-              const int tap = kk / ca.C, cc = kk - tap * ca.C;
-              const int ty = tap / ca.k, tx_ = tap - ty * ca.k;
-              tma_load_4d(sA + s * A_BYTES + j * (64 * ca.cbw * 2), &mapA, &ctl.full[s], cc,
-                          tx_ - ca.p, oy * ca.s - ca.p + ty, im);
-            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (j < nbox)
+                tma_load_4d(sA + s * A_BYTES + j * (64 * ca.cbw * 2), &mapA, &ctl.full[s], bc[j], bx[j],
+                            oy * ca.s + by[j], im);
 #pragma unroll
             for (int j = 0; j < BN / 64; ++j)
               tma_load_2d(sB + s * B_BYTES + j * 8192, &mapB, &ctl.full[s], n0 + 64 * j, k);
@@ -444,6 +457,11 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
           }
         }
         __syncwarp();
+        if (ca.on == 2) {  // the next 64 pixels: whole output rows, or whole images
+          oy += wg_rows;
+          im += wg_imgs;
+          if (oy >= ca.Ho) { oy = 0; ++im; }
+        }
         if ((c0 += kstep) == ca.C) {
           c0 = 0;
           if (++kx == ca.k) { kx = 0; ++ky; }
