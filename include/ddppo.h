@@ -506,10 +506,11 @@ int ddppo_conv2d_e4m3(int32_t N, int32_t H, int32_t W, int32_t C, int32_t Cout, 
 int ddppo_group_norm(int32_t N, int32_t HW, int32_t C, const float* z, const float* gamma,
                      const float* beta, const float* resid, int32_t relu, float* out, float* mean,
                      float* rstd, void* stream);
-/* How the encoder's forward GroupNorms run. An image of at most 32K elements is summed by
- * one block: with at least 4 images per SM the same block then normalises it (one launch,
- * the image re-read from L2); with fewer, a second launch normalises it, spread over many
- * blocks. A larger
+/* How the encoder's forward GroupNorms run. With fewer than 4 images per SM, images of at
+ * most 32K elements are cut into slices of channels, each summed and normalised by one block
+ * (one launch) where the slices' shapes allow it, otherwise an image is summed by one block
+ * and normalised by a second launch over many. With more, one block sums and normalises an
+ * image (one launch, the image re-read from L2). A larger
  * image is split over S blocks: with on = 1 (the default) the statistics and the
  * normalisation run in one cooperative launch wherever every block fits on the GPU at once
  * (the image's blocks meet at a bounded per-image barrier, then normalise the rows they

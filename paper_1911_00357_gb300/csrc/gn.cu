@@ -308,17 +308,21 @@ __device__ __forceinline__ float finish_vec(const GNApply& a, const ChannelParam
 // sz, sd: the rows of z and of zd (else the residual) staged in shared memory, pitch Cs (null:
 // read from global memory).
 constexpr int kRows = 4;
-template <int V, bool RES, bool ZD>
+// blocks an SM of gn_image_kernel: four with kRows rows in flight where the images are many
+// waves; six with one row where they fit in one (700 images of 1024 x 32 with a residual: 65 us,
+// 78 in two waves of four)
+constexpr int kImageCtas = 4, kFewCtas = 6;
+template <int V, bool RES, bool ZD, int ROWS>
 __device__ __forceinline__ float normalise_rows(const GNApply& a, size_t ib, int pr, int end, int P, int C,
                                                 int c0, const float* sz, const float* sd, int Cs,
                                                 const float* mu, const float* rs, const float* mud,
                                                 const float* rsd, float f8s) {
   const ChannelParams<V, ZD> q(a, c0);
   float f8m = 0.f;
-  for (int p0 = pr; p0 < end; p0 += kRows * P) {
-    float x[kRows][V], r[kRows][V], d[kRows][V];
+  for (int p0 = pr; p0 < end; p0 += ROWS * P) {
+    float x[ROWS][V], r[ROWS][V], d[ROWS][V];
 #pragma unroll
-    for (int u = 0; u < kRows; ++u) {
+    for (int u = 0; u < ROWS; ++u) {
       const int p = p0 + u * P;
       if (p >= end) break;
       const size_t o = ib + (size_t)p * C + c0;
@@ -327,7 +331,7 @@ __device__ __forceinline__ float normalise_rows(const GNApply& a, size_t ib, int
       if (ZD) ldv<V>(sd ? sd + (size_t)p * Cs : a.zd + o, d[u]);
     }
 #pragma unroll
-    for (int u = 0; u < kRows; ++u) {
+    for (int u = 0; u < ROWS; ++u) {
       const int p = p0 + u * P;
       if (p >= end) break;
       f8m = fmaxf(f8m, finish_vec<V, RES, ZD>(a, q, ib + (size_t)p * C + c0, x[u], r[u], d[u], mu, rs, mud,
@@ -337,15 +341,15 @@ __device__ __forceinline__ float normalise_rows(const GNApply& a, size_t ib, int
   return f8m;
 }
 
-template <int V>
+template <int V, int ROWS, int ROWS2 = ROWS>  // ROWS2: with a second or third input
 __device__ __forceinline__ float normalise_rows_any(const GNApply& a, size_t ib, int pr, int end, int P, int C,
                                                     int c0, const float* sz, const float* sd, int Cs,
                                                     const float* mu, const float* rs, const float* mud,
                                                     const float* rsd, float f8s) {
-  if (a.zd && a.resid) return normalise_rows<V, true, true>(a, ib, pr, end, P, C, c0, sz, sd, Cs, mu, rs, mud, rsd, f8s);
-  if (a.zd) return normalise_rows<V, false, true>(a, ib, pr, end, P, C, c0, sz, sd, Cs, mu, rs, mud, rsd, f8s);
-  if (a.resid) return normalise_rows<V, true, false>(a, ib, pr, end, P, C, c0, sz, sd, Cs, mu, rs, mud, rsd, f8s);
-  return normalise_rows<V, false, false>(a, ib, pr, end, P, C, c0, sz, sd, Cs, mu, rs, mud, rsd, f8s);
+  if (a.zd && a.resid) return normalise_rows<V, true, true, ROWS2>(a, ib, pr, end, P, C, c0, sz, sd, Cs, mu, rs, mud, rsd, f8s);
+  if (a.zd) return normalise_rows<V, false, true, ROWS2>(a, ib, pr, end, P, C, c0, sz, sd, Cs, mu, rs, mud, rsd, f8s);
+  if (a.resid) return normalise_rows<V, true, false, ROWS2>(a, ib, pr, end, P, C, c0, sz, sd, Cs, mu, rs, mud, rsd, f8s);
+  return normalise_rows<V, false, false, ROWS>(a, ib, pr, end, P, C, c0, sz, sd, Cs, mu, rs, mud, rsd, f8s);
 }
 
 template <int V>
@@ -456,7 +460,8 @@ __global__ void __launch_bounds__(kThreads, kFusedBlocks) gn_fused_kernel(GNAppl
   const int R = C / V, P = blockDim.x / R;
   const int cv = threadIdx.x % R, pr = threadIdx.x / R, c0 = cv * V;
   const float f8s = a.out_f8 ? *a.f8_scale : 1.f;
-  const float f8m = normalise_rows_any<V>(a, ib, pb + pr, pe, P, C, c0, nullptr, nullptr, 0, st + c0 / 2, st + G + c0 / 2,
+  // with a residual two rows in flight: 95 us for 256 images of 4096 x 32, four rows 104
+  const float f8m = normalise_rows_any<V, kRows, 2>(a, ib, pb + pr, pe, P, C, c0, nullptr, nullptr, 0, st + c0 / 2, st + G + c0 / 2,
                           st + 2 * G + c0 / 2, st + 3 * G + c0 / 2, f8s);
   if (a.out_f8) block_amax(f8m, a.f8_amax);
 }
@@ -475,8 +480,8 @@ __device__ __forceinline__ void combine_groups_one(const float* p, const float* 
   }
 }
 
-template <int V, bool RES, bool ZD>
-__global__ void __launch_bounds__(kThreads, 4) gn_image_kernel(GNApply a, PixelCount px, int C, float eps) {
+template <int V, bool RES, bool ZD, int CTAS>
+__global__ void __launch_bounds__(kThreads, CTAS) gn_image_kernel(GNApply a, PixelCount px, int C, float eps) {
   DDPPO_PDL_ENTRY();
   extern __shared__ float sh[];
   const int HW = px.HW, n = blockIdx.x, G = C / 2;
@@ -504,13 +509,19 @@ __global__ void __launch_bounds__(kThreads, 4) gn_image_kernel(GNApply a, PixelC
   const int R = C / V, P = blockDim.x / R;
   const int cv = threadIdx.x % R, pr = threadIdx.x / R, c0 = cv * V;
   const float f8s = a.out_f8 ? *a.f8_scale : 1.f;
-  const float f8m = normalise_rows<V, RES, ZD>(a, ib, pr, HW, P, C, c0, nullptr, nullptr, 0, st + c0 / 2, st + G + c0 / 2,
+  const float f8m = normalise_rows<V, RES, ZD, CTAS == kImageCtas ? kRows : 1>(a, ib, pr, HW, P, C, c0, nullptr, nullptr, 0, st + c0 / 2, st + G + c0 / 2,
                           st + 2 * G + c0 / 2, st + 3 * G + c0 / 2, f8s);
   if (a.out_f8) block_amax(f8m, a.f8_amax);
 }
 
 // ---- backward reductions: g = dy (masked by relu_y > 0), xhat = (z - mu) rstd;
 //      per image and channel sum(g) and sum(g xhat); group means of gamma-weighted sums ----
+template <int V, int CTAS>
+void (*image_kernel(const GNApply& a))(GNApply, PixelCount, int, float) {
+  if (a.resid) return a.zd ? gn_image_kernel<V, true, true, CTAS> : gn_image_kernel<V, true, false, CTAS>;
+  return a.zd ? gn_image_kernel<V, false, true, CTAS> : gn_image_kernel<V, false, false, CTAS>;
+}
+
 template <int V>
 __global__ void __launch_bounds__(kThreads) gn_bwd_reduce_kernel(GNBack b, int HW, int C, int S,
                                                                  float* __restrict__ part,
@@ -747,7 +758,7 @@ __global__ void __launch_bounds__(kThreads) gn_slice_kernel(GNApply a, PixelCoun
     }
   }
   const float f8s = a.out_f8 ? *a.f8_scale : 1.f;
-  const float f8m = normalise_rows_any<4>(a, ib, pr, HW, P, C, c0, sz + cv * 4, sd + cv * 4, Cs, st + cv * 2,
+  const float f8m = normalise_rows_any<4, kRows>(a, ib, pr, HW, P, C, c0, sz + cv * 4, sd + cv * 4, Cs, st + cv * 2,
                           st + Gs + cv * 2, st + 2 * Gs + cv * 2, st + 3 * Gs + cv * 2, f8s);
   if (a.out_f8) block_amax(f8m, a.f8_amax);
 }
@@ -1185,12 +1196,10 @@ int launch_gn_fused(const GNApply& a, int N, int HW, int C, float eps, const GnS
     if (N < 4 * num_sms_cached()) return DDPPO_OK;
     const size_t smem = ((size_t)th * 2 * V + 6 * (size_t)C) * sizeof(float);
     const PixelCount px = pixel_count(HW);
-    if (V != 4) ::ddppo::launch_k(a.resid ? (a.zd ? gn_image_kernel<2, true, true> : gn_image_kernel<2, true, false>)
-                                          : (a.zd ? gn_image_kernel<2, false, true> : gn_image_kernel<2, false, false>),
-                                  N, th, smem, s, a, px, C, eps);
-    else ::ddppo::launch_k(a.resid ? (a.zd ? gn_image_kernel<4, true, true> : gn_image_kernel<4, true, false>)
-                                   : (a.zd ? gn_image_kernel<4, false, true> : gn_image_kernel<4, false, false>),
-                           N, th, smem, s, a, px, C, eps);
+    const auto kern = V != 4 ? image_kernel<2, kImageCtas>(a)
+                      : N <= kFewCtas * num_sms_cached() ? image_kernel<4, kFewCtas>(a)
+                                                         : image_kernel<4, kImageCtas>(a);
+    ::ddppo::launch_k(kern, N, th, smem, s, a, px, C, eps);
     DDPPO_CHECK_LAUNCH();
     *launched = true;
     return DDPPO_OK;
