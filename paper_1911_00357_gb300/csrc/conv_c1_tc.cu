@@ -1,5 +1,5 @@
-// Single-channel convolution on tcgen05 -- the encoder's stem (App. "Visual Encoder": a
-// 7x7 / stride-2 convolution of the 1-channel depth image) -- without an im2col matrix.
+// Single-channel convolution on tcgen05 without an im2col matrix, for the filters, strides and
+// sizes that the stem's own kernel (conv_stem.cu) does not take.
 //
 // A tile is 128 consecutive output pixels (NHWC order). Its patches (k x k taps of the one
 // input channel, zero outside the image and past k^2, 64 taps per row) are gathered by the
