@@ -11,6 +11,7 @@
 // (normalise + residual + ReLU, and the input gradient) are vectorised the same way.
 #include <algorithm>
 
+#include "gn_ring.cuh"
 #include "nn_kernels.cuh"
 #include "tc_common.cuh"
 
@@ -18,7 +19,7 @@ namespace ddppo {
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = kGnThreads;
 
 template <int V>
 __device__ __forceinline__ void ldv(const float* p, float (&v)[V]) {
@@ -75,10 +76,7 @@ __device__ __forceinline__ void stv_op(void* p, size_t i, const float (&v)[V], b
 }
 
 // threads of the block: R = C / V per pixel row, P rows per pass
-__host__ __device__ inline int rows_per_pass(int C, int V) {
-  const int R = C / V;
-  return R >= kThreads ? 1 : kThreads / R;
-}
+__host__ __device__ inline int rows_per_pass(int C, int V) { return gn_rows_per_pass(C, V); }
 
 // sums the per-thread pair (a[v], b[v]) over the P rows of the block for every channel,
 // in row order; results for channel c at out[2c], out[2c + 1]. sh holds blockDim x 2V.
@@ -849,7 +847,7 @@ __global__ void __launch_bounds__(kThreads) gn_bwd_slice_kernel(GNBack b, int HW
 // block per image and the same masks (6.3 ms when the masks were read from the stored fp32
 // outputs). Two blocks and two rows a thread: 4 rows 4.8 ms, three blocks 4.4, one row 4.7,
 // one block of 4 rows 4.1.
-constexpr int kRingThreads = 288, kRingCtas = 2, kRingMax = 6, kRingRows = 2;
+constexpr int kRingThreads = 288, kRingCtas = 2, kRingMax = 6;
 constexpr int kRingHalf = kRingRows * 4 * 1024, kRingUnit = 2 * kRingHalf + kRingRows * 256;
 __device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -1032,8 +1030,8 @@ size_t ring_smem(int units, int C) {
 int ring_units(const GNBack& b, int HW, int C) {
   const int kind = mask_kind(b, 4);
   if (C % 4 || C > 512 || kind == MASK_Y) return 0;
-  // the mask bits' copies move 16-byte multiples
-  if (kind == MASK_POS && (HW * C % 64 || rows_per_pass(C, 4) * C % 16)) return 0;
+  // other widths take the one-block-per-image form, whose threads load their own mask byte
+  if (kind == MASK_POS && !ring_mask_copies_ok(HW, C)) return 0;
   const size_t room = (size_t)228 * 1024 / kRingCtas - 2048 - ring_smem(0, C);
   return (int)std::min<size_t>(kRingMax, room / kRingUnit);
 }
