@@ -2,6 +2,7 @@
 // that complete the receiver's mbarrier, and the bounded wait for them (sm_103a).
 #pragma once
 
+#include "cluster_steps.cuh"
 #include "tc_common.cuh"
 
 namespace ddppo {
@@ -63,14 +64,32 @@ __device__ __forceinline__ void send4(uint32_t raddr, float v, uint32_t rbar) {
                : "memory");
 }
 
-// after the last step: every CTA of the cluster has issued all it sends; if one gave up,
-// let what is in flight land (bounded) before the shared memory goes away
-__device__ __forceinline__ void cluster_end(uint64_t* full, bool failed) {
+// After the last step. Every CTA tells the others the last step it sent and meets them: what
+// is sent from here on is nothing. A CTA that gave up in step t may still be written to: its
+// peers have sent step t, and those that had received all of it step t + 1. It waits (bounded)
+// for these blocks before its shared memory goes away, counting the blocks that never come as
+// delivered, so that the phase completes with the last one in flight.
+constexpr int kClusterMax = 16;
+__device__ __forceinline__ void cluster_end(uint64_t* full, int* sent, int ctas, int t, int T,
+                                            uint32_t cta_bytes, bool failed) {
+  __syncwarp();
+  if ((int)threadIdx.x < ctas)
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
+                     map_rank(smem_addr(&sent[cluster_rank()]), threadIdx.x)),
+                 "r"(min(t, T - 1))
+                 : "memory");
   __syncwarp();
   cluster_sync();
-  if (failed && threadIdx.x == 0) {
-    mbar_drain_wait(&full[0], 0u);
-    mbar_drain_wait(&full[1], 0u);
+  if (!failed || threadIdx.x != 0) return;
+  for (int s = t; s <= t + 1; ++s) {
+    const int missing = step_missing(sent, ctas, s, T);
+    if (missing < 0) continue;
+    uint64_t* bar = &full[step_bar(s)];
+    if (missing)
+      asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)),
+                   "r"(missing * cta_bytes)
+                   : "memory");
+    mbar_drain_wait(bar, step_parity(s));
   }
 }
 

@@ -30,8 +30,9 @@
 // stores.
 //
 // Every wait is bounded: on a run-out the sticky timeout flag is set, the CTA sends and
-// stores nothing more, and every CTA meets the cluster barrier at the end before its shared
-// memory is released.
+// stores nothing more, and every CTA meets the cluster barrier at the end; one that gave up
+// then waits (bounded) for the blocks still on their way to it before its shared memory is
+// released.
 #include <algorithm>
 #include <atomic>
 
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_fwd_kernel(LstmCl a) {
   __shared__ __align__(128) uint8_t hs[2][CL * LC_BLOCK];
   __shared__ __align__(16) uint8_t stage[2][LC_BLOCK];
   __shared__ uint64_t full[2];
+  __shared__ int sent[kClusterMax];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
   const int cta = (int)cluster_rank();
   const int e0 = (int)(blockIdx.x / CL) * a.epc, ne = min(a.epc, a.E - e0);
@@ -140,9 +142,10 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_fwd_kernel(LstmCl a) {
   cluster_sync();  // every barrier is initialised and every buffer zeroed before a send
 
   bool ok = true;
-  for (int t = 0; t < a.T; ++t) {
-    if (t > 0) ok = wait_bytes(&full[t & 1], (uint32_t)((t - 1) >> 1) & 1u, a.err) && ok;
-    if (threadIdx.x == 0 && t > 0 && t + 2 < a.T)
+  int t = 0;
+  for (; t < a.T; ++t) {
+    if (t > 0) ok = wait_bytes(&full[step_bar(t)], step_parity(t), a.err) && ok;
+    if (threadIdx.x == 0 && ok && t > 0 && t + 2 < a.T)
       expect_bytes(&full[t & 1], (uint32_t)(CL * ne * 64));
     // the next step's input projection and mask, in flight during this step's MMAs
     float gn[4] = {0.f, 0.f, 0.f, 0.f};
@@ -231,7 +234,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_fwd_kernel(LstmCl a) {
     for (int q = 0; q < 4; ++q) gx[q] = gn[q];
     mk = mn;
   }
-  cluster_end(full, !ok);
+  cluster_end(full, sent, CL, t, a.T, (uint32_t)(ne * 64), !ok);
 }
 
 // back-propagation: CTA j owns units [32 j, 32 j + 32), i.e. rows of W_hh^T [H, 4H]. The
@@ -246,6 +249,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_bwd_kernel(LstmCl a) {
   __shared__ __align__(16) uint8_t stage[4 * LC_BLOCK];
   __shared__ float red[8][LC_ENVS][LC_RED_PITCH];
   __shared__ uint64_t full[2];
+  __shared__ int sent[kClusterMax];
   constexpr int BUF = CL * 4 * LC_BLOCK;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
   const int cta = (int)cluster_rank();
@@ -286,7 +290,8 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_bwd_kernel(LstmCl a) {
   cluster_sync();
 
   bool ok = true;
-  for (int it = 0; it < a.T; ++it) {
+  int it = 0;
+  for (; it < a.T; ++it) {
     const int t = a.T - 1 - it;
     // forward values of the step, in flight during the wait and the MMAs
     float gt[4] = {0.f, 0.f, 0.f, 0.f}, cprev = 0.f, dha = 0.f;
@@ -301,8 +306,8 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_bwd_kernel(LstmCl a) {
     }
     float rec = 0.f;
     if (it > 0) {
-      ok = wait_bytes(&full[it & 1], (uint32_t)((it - 1) >> 1) & 1u, a.err) && ok;
-      if (threadIdx.x == 0 && it + 2 < a.T) expect_bytes(&full[it & 1], bytes);
+      ok = wait_bytes(&full[step_bar(it)], step_parity(it), a.err) && ok;
+      if (threadIdx.x == 0 && ok && it + 2 < a.T) expect_bytes(&full[it & 1], bytes);
       float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
       // slice = gate warp / 2, units of CTAs (warp % 2) CL / 2 ..
       const uint32_t db = smem_addr(ds + (it & 1) * BUF) + (uint32_t)ldsm_off(lane) +
@@ -371,7 +376,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl_bwd_kernel(LstmCl a) {
       }
     }
   }
-  cluster_end(full, !ok);
+  cluster_end(full, sent, CL, it, a.T, (uint32_t)(4 * ne * 64), !ok);
 }
 
 // ---- FP32 operands: the same scheme on the CUDA cores ----
@@ -409,6 +414,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl32_fwd_kernel(LstmCl a) 
   __shared__ __align__(16) float hs[2][LC_ENVS][H];
   __shared__ float red[8][LC_ENVS][LC_UNITS];
   __shared__ uint64_t full[2];
+  __shared__ int sent[kClusterMax];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cta = (int)cluster_rank();
   const int e0 = (int)(blockIdx.x / CL) * a.epc, ne = min(a.epc, a.E - e0);
@@ -443,9 +449,10 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl32_fwd_kernel(LstmCl a) 
   cluster_sync();
 
   bool ok = true;
-  for (int t = 0; t < a.T; ++t) {
-    if (t > 0) ok = wait_bytes(&full[t & 1], (uint32_t)((t - 1) >> 1) & 1u, a.err) && ok;
-    if (threadIdx.x == 0 && t > 0 && t + 2 < a.T) expect_bytes(&full[t & 1], bytes);
+  int t = 0;
+  for (; t < a.T; ++t) {
+    if (t > 0) ok = wait_bytes(&full[step_bar(t)], step_parity(t), a.err) && ok;
+    if (threadIdx.x == 0 && ok && t > 0 && t + 2 < a.T) expect_bytes(&full[t & 1], bytes);
     const bool last = t + 1 == a.T;
     float gn[4] = {0.f, 0.f, 0.f, 0.f};
     bool mn = false;
@@ -485,7 +492,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl32_fwd_kernel(LstmCl a) 
     for (int q = 0; q < 4; ++q) gx[q] = gn[q];
     mk = mn;
   }
-  cluster_end(full, !ok);
+  cluster_end(full, sent, CL, t, a.T, (uint32_t)(LC_UNITS * ne * 4), !ok);
 }
 
 template <int H>
@@ -495,6 +502,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl32_bwd_kernel(LstmCl a) 
   extern __shared__ __align__(128) float dz_in[];  // [2][LC_ENVS][4H]
   __shared__ float red[8][LC_ENVS][LC_UNITS];
   __shared__ uint64_t full[2];
+  __shared__ int sent[kClusterMax];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cta = (int)cluster_rank();
   const int e0 = (int)(blockIdx.x / CL) * a.epc, ne = min(a.epc, a.E - e0);
@@ -518,7 +526,8 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl32_bwd_kernel(LstmCl a) 
   cluster_sync();
 
   bool ok = true;
-  for (int it = 0; it < a.T; ++it) {
+  int it = 0;
+  for (; it < a.T; ++it) {
     const int t = a.T - 1 - it;
     float gt[4] = {0.f, 0.f, 0.f, 0.f}, cprev = 0.f, dha = 0.f;
     bool mk = false;
@@ -532,8 +541,8 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl32_bwd_kernel(LstmCl a) 
     }
     float rec = 0.f;
     if (it > 0) {
-      ok = wait_bytes(&full[it & 1], (uint32_t)((it - 1) >> 1) & 1u, a.err) && ok;
-      if (threadIdx.x == 0 && it + 2 < a.T) expect_bytes(&full[it & 1], bytes);
+      ok = wait_bytes(&full[step_bar(it)], step_parity(it), a.err) && ok;
+      if (threadIdx.x == 0 && ok && it + 2 < a.T) expect_bytes(&full[it & 1], bytes);
       const float* in = dz_in + (size_t)(it & 1) * LC_ENVS * ROW + warp * K2;
       for (int n = 0; n < ne; ++n) red[warp][n][lane] = dot_row<K2>(w, in + n * ROW);
       if (__syncthreads_or(ok ? 0 : 1)) { ok = false; break; }
@@ -568,7 +577,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) lstm_cl32_bwd_kernel(LstmCl a) 
       ((float*)a.dg_op)[gb + q * H] = dz[q];
     }
   }
-  cluster_end(full, !ok);
+  cluster_end(full, sent, CL, it, a.T, (uint32_t)(4 * LC_UNITS * ne * 4), !ok);
 }
 
 typedef void (*ClKernel)(LstmCl);
