@@ -22,6 +22,10 @@
  *     stream. Work is enqueued asynchronously on it; results are ready when the
  *     stream is synchronised. Entry points that enqueue work never allocate or
  *     synchronise, so they can be captured into a CUDA graph, except where noted.
+ *     The calls without a context may run on several streams and threads at once (but for
+ *     ddppo_ppo_loss_static): the scratch of those that need some belongs to the stream (the
+ *     first such call on a stream allocates it; beyond 16 streams of a device, and in a
+ *     capture, it is stream-ordered memory of that call, part of the graph).
  *   - Arrays are dense, row-major, time-major where a time axis exists.
  *   - Units of the world: positions in u = 1e-4 m (int32), depth in metres.
  *   - Errors detected on the device (an index outside a buffer, a capped wait
@@ -442,8 +446,7 @@ int ddppo_load(ddppo_ctx* ctx, const ddppo_rollout* ro, const char* path, void* 
  * tcgen05 tensor-core path with fp32 accumulation when rows are 16-byte aligned). C [dev]
  * row-major fp32, or bf16 when c_bf16 (then beta must be 0). bias [dev] [N] or NULL.
  * status [dev] int32 or NULL receives the sticky timeout flag (2) of a bounded
- * tensor-core wait. The first call per device allocates a split-K workspace (not
- * capturable). */
+ * tensor-core wait. Split-K sums take 64 MB of the stream's scratch. */
 int ddppo_gemm(int32_t M, int32_t N, int32_t K, int32_t op_bf16, const void* A, int32_t lda,
                int32_t a_t, const void* B, int32_t ldb, int32_t b_t, void* C, int32_t ldc,
                int32_t c_bf16, float beta, const float* bias, int32_t relu, int32_t* status,
@@ -460,8 +463,7 @@ int ddppo_gemm(int32_t M, int32_t N, int32_t K, int32_t op_bf16, const void* A, 
  * p = k / 2, C == 32, Cout <= 128 and W + 2p <= 256, or -- the encoder's stem -- C == 1,
  * k * k <= 64 and Cout 16, 32 or 64 (each 128-pixel tile's patches gathered by the CTA
  * into shared memory, the weights resident; at most 2^30 output pixels); E_CONFIG
- * otherwise. status as for ddppo_gemm. The first call per device allocates a split-K
- * workspace. */
+ * otherwise. status and scratch as for ddppo_gemm. */
 int ddppo_conv2d(int32_t N, int32_t H, int32_t W, int32_t C, int32_t Cout, int32_t k,
                  int32_t stride, int32_t pad, const void* x, const void* w, float* y,
                  float beta, int32_t* status, void* stream);
@@ -472,8 +474,8 @@ int ddppo_conv2d(int32_t N, int32_t H, int32_t W, int32_t C, int32_t Cout, int32
  * filter tap with a 4-D TMA copy. x [dev] NHWC bf16 [N, H, W, C]; dy [dev] bf16
  * [N, Ho, Wo, Cout]; dw [dev] fp32 [Cout, k*k*C]. Requires C == 32 or C % 64 == 0,
  * Cout % 8 == 0, an output width dividing 64 and whole 64-pixel blocks (Ho*Wo a multiple
- * of 64 made of whole rows, or a divisor of 64); E_CONFIG otherwise. status and the
- * workspace as for ddppo_conv2d. */
+ * of 64 made of whole rows, or a divisor of 64); E_CONFIG otherwise. status and scratch
+ * as for ddppo_gemm. */
 int ddppo_conv2d_wgrad(int32_t N, int32_t H, int32_t W, int32_t C, int32_t Cout, int32_t k,
                        int32_t stride, int32_t pad, const void* x, const void* dy, float* dw,
                        float beta, int32_t* status, void* stream);
@@ -502,7 +504,7 @@ int ddppo_conv2d_e4m3(int32_t N, int32_t H, int32_t W, int32_t C, int32_t Cout, 
  * groups of 2 channels, eps 1e-5): out = act(gn(z) gamma + beta + resid) over NHWC z [dev]
  * fp32 [N, HW, C]; gamma, beta [dev] [C]; resid [dev] [N, HW, C] or NULL; relu 0/1; mean,
  * rstd [dev] [N, C/2] receive the group statistics. N <= 8192, C even <= 1024 (E_ARG
- * otherwise). The first call per device allocates a scratch (not capturable). */
+ * otherwise). 78 MB of the stream's scratch. */
 int ddppo_group_norm(int32_t N, int32_t HW, int32_t C, const float* z, const float* gamma,
                      const float* beta, const float* resid, int32_t relu, float* out, float* mean,
                      float* rstd, void* stream);
@@ -523,8 +525,8 @@ int ddppo_group_norm_one_launch(ddppo_ctx* ctx, int32_t on);
  * convolution; squeeze-and-excitation), stand-alone, fp32 NHWC:
  * ddppo_grouped_conv3x3: z [dev] [N, Ho, Wo, C] = the 3x3 convolution, padding 1, of x
  * [dev] [N, H, W, C] with `groups` groups, weights w [dev] [C, C/groups, 3, 3] (PyTorch's
- * grouped layout); C / groups <= 16, C <= 1024, stride 1 or 2 (E_ARG otherwise); the first
- * call per device allocates a weight scratch (not capturable).
+ * grouped layout); C / groups <= 16, C <= 1024, stride 1 or 2 (E_ARG otherwise); the
+ * weights' layout takes 0.6 MB of the stream's scratch.
  * ddppo_squeeze_excite: for u [dev] [N, HW, C]: m = mean_hw u [N, C], a = relu(W1 m + b1)
  * [N, Cr], gate = sigmoid(W2 a + b2) [N, C], y = relu(u gate + sc) [N, HW, C] (sc [dev] or
  * NULL); W1 [Cr, C], b1 [Cr], W2 [C, Cr], b2 [C]; every output [dev]. */

@@ -9,6 +9,7 @@
 #include "net.cuh"
 #include "nn_kernels.cuh"
 #include "rl.cuh"
+#include "scratch.cuh"
 
 namespace ddppo {
 // infer: an act-time pass (policy_act, the collect loop, the bootstrap value); under FP8
@@ -722,6 +723,19 @@ extern "C" int ddppo_count_kernels(ddppo_ctx* x, const ddppo_rollout* ro,
   return rc;
 }
 
+// split-K sums of a stand-alone contraction on stream s; scratch holds them for the call
+static int standalone_ws(GemmWorkspace* ws, Scratch* scratch, int32_t* status, cudaStream_t s) {
+  const size_t elems = (size_t)16 << 20;
+  DDPPO_TRY(scratch->take(SCRATCH_SPLITK, elems * sizeof(float), 0, s));
+  ws->partial = scratch->as<float>();
+  ws->partial_elems = elems;
+  int dev = 0;
+  DDPPO_CHECK_CUDA(cudaGetDevice(&dev));
+  cudaDeviceGetAttribute(&ws->num_sms, cudaDevAttrMultiProcessorCount, dev);
+  ws->err = status;
+  return DDPPO_OK;
+}
+
 // ---- stand-alone GEMM (the contraction every network layer uses) ----
 extern "C" int ddppo_gemm(int32_t M, int32_t N, int32_t K, int32_t op_bf16, const void* A,
                           int32_t lda, int32_t a_t, const void* B, int32_t ldb, int32_t b_t,
@@ -732,17 +746,9 @@ extern "C" int ddppo_gemm(int32_t M, int32_t N, int32_t K, int32_t op_bf16, cons
   ARG(A && B && C, "gemm: null argument");
   ARG(lda >= (a_t ? M : K) && ldb >= (b_t ? N : K) && ldc >= N,
       "gemm: leading dimension smaller than the row");
-  static float* partial[64] = {};
-  int dev = 0;
-  DDPPO_CHECK_CUDA(cudaGetDevice(&dev));
-  ARG(dev < 64, "gemm: device ordinal out of range");
-  const size_t elems = (size_t)16 << 20;
-  if (!partial[dev]) DDPPO_CHECK_CUDA(cudaMalloc(&partial[dev], elems * sizeof(float)));
+  Scratch scratch;
   GemmWorkspace ws;
-  ws.partial = partial[dev];
-  ws.partial_elems = elems;
-  cudaDeviceGetAttribute(&ws.num_sms, cudaDevAttrMultiProcessorCount, dev);
-  ws.err = status;
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
   GemmDesc d;
   d.M = M; d.N = N; d.K = K; d.A = A; d.lda = lda; d.B = B; d.ldb = ldb; d.C = C; d.ldc = ldc;
   d.c_bf16 = c_bf16; d.beta = beta; d.bias = bias; d.relu = relu;
@@ -817,29 +823,23 @@ extern "C" int ddppo_group_norm(int32_t N, int32_t HW, int32_t C, const float* z
   ARG(N >= 1 && N <= 8192 && HW >= 1 && C >= 2 && C <= 1024 && C % 2 == 0,
       "group_norm: N in [1, 8192], C even in [2, 1024]");
   ARG(z && gamma && beta && out && mean && rstd, "group_norm: null argument");
-  int dev = 0;
-  DDPPO_CHECK_CUDA(cudaGetDevice(&dev));
-  ARG(dev < 64, "group_norm: device ordinal out of range");
-  static GnScratch ws[64];
-  if (!ws[dev].part) {
-    GnScratch w;
-    w.max_images = 8192;
-    w.part_elems = gn_part_elems(w.max_images, 1024);
-    DDPPO_CHECK_CUDA(cudaMalloc(&w.part, w.part_elems * sizeof(float)));
-    DDPPO_CHECK_CUDA(cudaMalloc(&w.cnt, (size_t)w.max_images * sizeof(int)));
-    DDPPO_CHECK_CUDA(cudaMemset(w.cnt, 0, (size_t)w.max_images * sizeof(int)));
-    DDPPO_CHECK_CUDA(cudaMalloc(&w.cnt2, (size_t)w.max_images * sizeof(int)));
-    DDPPO_CHECK_CUDA(cudaMemset(w.cnt2, 0, (size_t)w.max_images * sizeof(int)));
-    ws[dev] = w;
-  }
   cudaStream_t s = (cudaStream_t)stream;
+  GnScratch w;
+  w.max_images = 8192;
+  w.part_elems = gn_part_elems(w.max_images, 1024);
+  const size_t part = w.part_elems * sizeof(float), cnts = (size_t)w.max_images * sizeof(int);
+  Scratch scratch;
+  DDPPO_TRY(scratch.take(SCRATCH_GN, part + 2 * cnts, 2 * cnts, s));
+  w.part = scratch.as<float>();
+  w.cnt = scratch.as<int>(part);
+  w.cnt2 = scratch.as<int>(part + cnts);
   GNApply a{};
   a.z = z; a.mean = mean; a.rstd = rstd; a.gamma = gamma; a.beta = beta;
   a.resid = resid; a.out = out; a.relu = relu ? 1 : 0;
   bool done = false;
-  DDPPO_TRY(launch_gn_fused(a, N, HW, C, 1e-5f, ws[dev], nullptr, s, &done));
+  DDPPO_TRY(launch_gn_fused(a, N, HW, C, 1e-5f, w, nullptr, s, &done));
   if (done) return DDPPO_OK;
-  DDPPO_TRY(launch_gn_stats(z, N, HW, C, 1e-5f, mean, rstd, ws[dev], s));
+  DDPPO_TRY(launch_gn_stats(z, N, HW, C, 1e-5f, mean, rstd, w, s));
   return launch_gn_apply(a, N, HW, C, s);
 }
 
@@ -857,17 +857,15 @@ extern "C" int ddppo_grouped_conv3x3(int32_t N, int32_t H, int32_t W, int32_t C,
           (stride == 1 || stride == 2) && C <= 1024,
       "grouped_conv3x3: bad sizes (C / groups <= 16, C <= 1024, stride 1 or 2)");
   ARG(x && w && z, "grouped_conv3x3: null argument");
-  int dev = 0;
-  DDPPO_CHECK_CUDA(cudaGetDevice(&dev));
-  ARG(dev < 64, "grouped_conv3x3: device ordinal out of range");
-  static float* wbuf[64] = {};
-  if (!wbuf[dev]) DDPPO_CHECK_CUDA(cudaMalloc(&wbuf[dev], (size_t)1024 * 16 * 9 * sizeof(float)));
   cudaStream_t s = (cudaStream_t)stream;
+  Scratch scratch;
+  DDPPO_TRY(scratch.take(SCRATCH_GCONV, (size_t)1024 * 16 * 9 * sizeof(float), 0, s));
+  float* wbuf = scratch.as<float>();
   GConv g;
   g.N = N; g.H = H; g.W = W; g.C = C; g.cpg = C / groups; g.s = stride;
   g.Ho = (H + 2 - 3) / stride + 1; g.Wo = (W + 2 - 3) / stride + 1;
-  DDPPO_TRY(launch_gconv_w_prep(w, C, g.cpg, wbuf[dev], false, s));
-  return launch_gconv_fwd(g, x, wbuf[dev], z, false, s);
+  DDPPO_TRY(launch_gconv_w_prep(w, C, g.cpg, wbuf, false, s));
+  return launch_gconv_fwd(g, x, wbuf, z, false, s);
 }
 
 extern "C" int ddppo_squeeze_excite(int32_t N, int32_t HW, int32_t C, int32_t Cr, const float* u,
@@ -884,20 +882,6 @@ extern "C" int ddppo_squeeze_excite(int32_t N, int32_t HW, int32_t C, int32_t Cr
 }
 
 // ---- stand-alone convolution on the implicit-im2col tensor-core path ----
-static int standalone_ws(GemmWorkspace* ws, int32_t* status) {
-  int dev = 0;
-  DDPPO_CHECK_CUDA(cudaGetDevice(&dev));
-  static float* partial[64] = {};
-  ARG(dev < 64, "conv2d: device ordinal out of range");
-  const size_t elems = (size_t)16 << 20;
-  if (!partial[dev]) DDPPO_CHECK_CUDA(cudaMalloc(&partial[dev], elems * sizeof(float)));
-  ws->partial = partial[dev];
-  ws->partial_elems = elems;
-  cudaDeviceGetAttribute(&ws->num_sms, cudaDevAttrMultiProcessorCount, dev);
-  ws->err = status;
-  return DDPPO_OK;
-}
-
 static int conv_args(int32_t N, int32_t H, int32_t W, int32_t C, int32_t Cout, int32_t k,
                      int32_t stride, int32_t pad, ConvShape* c) {
   ARG(N >= 1 && H >= 1 && W >= 1 && C >= 1 && Cout >= 1 && k >= 1 && stride >= 1 && pad >= 0,
@@ -922,8 +906,9 @@ extern "C" int ddppo_conv2d(int32_t N, int32_t H, int32_t W, int32_t C, int32_t 
     set_error("conv2d: shape not covered by the implicit-im2col path");
     return DDPPO_E_CONFIG;
   }
+  Scratch scratch;
   GemmWorkspace ws;
-  DDPPO_TRY(standalone_ws(&ws, status));
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
   GemmDesc d;
   d.M = N * c.Ho * c.Wo; d.N = Cout; d.K = k * k * C;
   d.conv = &c; d.A = x; d.lda = d.K; d.B = w; d.ldb = d.K;
@@ -946,15 +931,13 @@ extern "C" int ddppo_quantize_e4m3(const void* x, int32_t x_bf16, int64_t n, voi
                                    void* stream) {
   ARG(n >= 0, "quantize_e4m3: negative size");
   ARG(x && q && scale, "quantize_e4m3: null argument");
-  int dev = 0;
-  DDPPO_CHECK_CUDA(cudaGetDevice(&dev));
-  ARG(dev < 64, "quantize_e4m3: device ordinal out of range");
-  static unsigned* amax[64] = {};
-  if (!amax[dev]) DDPPO_CHECK_CUDA(cudaMalloc(&amax[dev], sizeof(unsigned)));
   cudaStream_t s = (cudaStream_t)stream;
-  DDPPO_CHECK_CUDA(cudaMemsetAsync(amax[dev], 0, sizeof(unsigned), s));
-  DDPPO_TRY(launch_amax(x, x_bf16 != 0, (size_t)n, amax[dev], s));
-  return launch_quant_e4m3(x, x_bf16 != 0, (size_t)n, amax[dev], scale, (uint8_t*)q, s);
+  Scratch scratch;
+  DDPPO_TRY(scratch.take(SCRATCH_AMAX, sizeof(unsigned), 0, s));
+  unsigned* amax = scratch.as<unsigned>();
+  DDPPO_CHECK_CUDA(cudaMemsetAsync(amax, 0, sizeof(unsigned), s));
+  DDPPO_TRY(launch_amax(x, x_bf16 != 0, (size_t)n, amax, s));
+  return launch_quant_e4m3(x, x_bf16 != 0, (size_t)n, amax, scale, (uint8_t*)q, s);
 }
 
 extern "C" int ddppo_gemm_e4m3(int32_t M, int32_t N, int32_t K, const void* A, int32_t lda,
@@ -965,8 +948,9 @@ extern "C" int ddppo_gemm_e4m3(int32_t M, int32_t N, int32_t K, const void* A, i
   if (M == 0 || N == 0) return DDPPO_OK;
   ARG(A && B && C, "gemm_e4m3: null argument");
   ARG(lda >= K && ldb >= K && ldc >= N, "gemm_e4m3: leading dimension smaller than the row");
+  Scratch scratch;
   GemmWorkspace ws;
-  DDPPO_TRY(standalone_ws(&ws, status));
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
   GemmDesc d;
   d.M = M; d.N = N; d.K = K; d.A = A; d.lda = lda; d.B = B; d.ldb = ldb; d.C = C; d.ldc = ldc;
   d.beta = beta; d.bias = bias; d.relu = relu;
@@ -982,8 +966,9 @@ extern "C" int ddppo_conv2d_e4m3(int32_t N, int32_t H, int32_t W, int32_t C, int
   DDPPO_TRY(conv_args(N, H, W, C, Cout, k, stride, pad, &c));
   ARG(x && w && y, "conv2d_e4m3: null argument");
   c.Cout = Cout;
+  Scratch scratch;
   GemmWorkspace ws;
-  DDPPO_TRY(standalone_ws(&ws, status));
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
   GemmDesc d;
   d.M = N * c.Ho * c.Wo; d.N = Cout; d.K = k * k * C;
   d.conv = &c; d.A = x; d.lda = d.K; d.B = w; d.ldb = d.K;
@@ -1004,8 +989,9 @@ extern "C" int ddppo_conv2d_wgrad(int32_t N, int32_t H, int32_t W, int32_t C, in
     set_error("conv2d_wgrad: shape not covered by the implicit weight-gradient path");
     return DDPPO_E_CONFIG;
   }
+  Scratch scratch;
   GemmWorkspace ws;
-  DDPPO_TRY(standalone_ws(&ws, status));
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
   GemmDesc d;
   d.M = Cout; d.N = k * k * C; d.K = N * c.Ho * c.Wo;
   d.A = dy; d.lda = Cout; d.a_t = 1;
