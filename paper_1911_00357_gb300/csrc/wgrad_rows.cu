@@ -22,7 +22,11 @@
 // Each CTA (one per SM: all of TMEM) accumulates every unit of its split of the job and
 // writes its sums once; a second kernel adds the splits in order. Rows past the last shift
 // of a box are zeros that no copy overwrites: they meet dz = 0, and stale values there could
-// be NaN.
+// be NaN. Pad anchors meet real pixels too (the last column through the left tap, the next
+// row's first through the right one, the last row through the upper one where a unit reaches
+// past the image): with dz = 0 that adds nothing unless the pixel is an infinity or a NaN, of
+// which 0 x makes a NaN. The second kernel therefore forms a sum that is not finite again, from
+// the pixels of its own tap alone.
 //
 // Measured (4096 images): 16x16, 64 -> 64 channels 106 us against 367 us for the gather form
 // (0.73 PFLOP/s; N = 64 leaves the MMAs bound by shared-memory reads); the seven
@@ -184,14 +188,44 @@ __global__ void __launch_bounds__(WR_THREADS, 1)
   }
 }
 
+// One weight's gradient from its own pixels alone, in plain order (zero outside the image).
+// Out of line and last in its caller: no stack frame there, 48 registers a thread (32 without
+// it) and the same time (97.2 us a call at 4096 x 16x16, 64 -> 64; 96.9).
+struct WrPixels {
+  const __nv_bfloat16* x;
+  const __nv_bfloat16* dz;
+  int N, H, W, C, Cout;
+};
+__device__ __noinline__ void wgrad_plain(const WrPixels& p, int ky, int kx, int ci, int co, float* d,
+                                         float beta) {
+  double sum = 0.0;
+  for (int r = 0; r < p.N * p.H; ++r) {
+    const int iy = r % p.H + ky - 1;
+    const bool in_row = iy >= 0 && iy < p.H;
+    const __nv_bfloat16* dz = p.dz + (size_t)r * p.W * p.Cout + co;
+    const __nv_bfloat16* x = p.x + ((size_t)(r + ky - 1) * p.W + kx - 1) * p.C + ci;
+    float row = 0.f;
+#pragma unroll 4
+    for (int c = 0; c < p.W; ++c) {
+      const bool in = in_row && c + kx >= 1 && c + kx <= p.W;
+      const float v = in ? __bfloat162float(x[(ptrdiff_t)c * p.C]) : 0.f;
+      row = fmaf(__bfloat162float(dz[(size_t)c * p.Cout]), v, row);
+    }
+    sum += row;
+    if (isnan(sum)) break;  // and stays so
+  }
+  const float t = (float)sum;
+  *d = beta != 0.f ? beta * *d + t : t;
+}
+
 // dw (+)= the splits' sums. A block takes 8 accumulator rows (input channels) x 32 columns
 // (output channels) of one accumulator of one job: 64 threads of 16-byte loads by 4 slices
 // of the splits, the slices added in order; 8 consecutive input channels are written
 // together.
 template <int NB>
 __global__ void __launch_bounds__(256) wgrad_rows_reduce_kernel(const float* __restrict__ part,
-                                                                WrArgs a, int C, float* __restrict__ dw,
-                                                                int ldw, float beta) {
+                                                                WrArgs a, const __grid_constant__ WrPixels px,
+                                                                float* __restrict__ dw, int ldw, float beta) {
   DDPPO_PDL_ENTRY();
   constexpr int NACC = NB == 64 ? 6 : 3;
   __shared__ float sh[4][8][33];
@@ -218,8 +252,9 @@ __global__ void __launch_bounds__(256) wgrad_rows_reduce_kernel(const float* __r
   } else {
     ky = job % 3; kx = q; ci = (job / 3) % a.cb128 * 128 + row; co = job / (3 * a.cb128) * 128 + c0 + n;
   }
-  float* d = dw + (size_t)co * ldw + (size_t)(ky * 3 + kx) * C + ci;
-  *d = beta != 0.f ? beta * *d + t : t;
+  float* d = dw + (size_t)co * ldw + (size_t)(ky * 3 + kx) * px.C + ci;
+  if (isfinite(t)) *d = beta != 0.f ? beta * *d + t : t;
+  else wgrad_plain(px, ky, kx, ci, co, d, beta);
 }
 
 // units, ring and shared memory for a convolution; false when it is not covered
@@ -280,7 +315,7 @@ bool wr_map(CUtensorMap* m, const void* p, int C, const ConvShape& c, int Wp, in
 }
 
 template <int NB>
-int launch_wr(const WrPlan& p, const CUtensorMap& mx, const CUtensorMap& md, const ConvShape& c,
+int launch_wr(const WrPlan& p, const CUtensorMap& mx, const CUtensorMap& md, const WrPixels& px,
               float* dw, int ldw, float beta, const GemmWorkspace& ws, cudaStream_t s) {
   static bool attr_done[64] = {};
   int dev = 0;
@@ -294,7 +329,7 @@ int launch_wr(const WrPlan& p, const CUtensorMap& mx, const CUtensorMap& md, con
                     ws.err);
   DDPPO_CHECK_LAUNCH();
   ::ddppo::launch_k(wgrad_rows_reduce_kernel<NB>, dim3(16 * (NB / 32), NB == 64 ? 6 : 3, p.jobs), 256, 0, s,
-                    ws.partial, p.a, c.C, dw, ldw, beta);
+                    ws.partial, p.a, px, dw, ldw, beta);
   DDPPO_CHECK_LAUNCH();
   return DDPPO_OK;
 }
@@ -328,8 +363,9 @@ int conv_wgrad_rows(const ConvShape& c, const void* x, const void* dz, float* dw
     set_error("wgrad_rows: tensor map encoding failed");
     return DDPPO_E_CUDA;
   }
-  if (p.nb == 64) return launch_wr<64>(p, mx, md, c, dw, ldw, beta, ws, s);
-  return launch_wr<128>(p, mx, md, c, dw, ldw, beta, ws, s);
+  const WrPixels px{(const __nv_bfloat16*)x, (const __nv_bfloat16*)dz, c.N, c.H, c.W, c.C, c.Cout};
+  if (p.nb == 64) return launch_wr<64>(p, mx, md, px, dw, ldw, beta, ws, s);
+  return launch_wr<128>(p, mx, md, px, dw, ldw, beta, ws, s);
 }
 
 }  // namespace ddppo
