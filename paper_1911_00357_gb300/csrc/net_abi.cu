@@ -902,6 +902,10 @@ extern "C" int ddppo_conv2d(int32_t N, int32_t H, int32_t W, int32_t C, int32_t 
   c.Cout = Cout;
   // one input channel (the encoder's stem): the contraction gathers its patches itself
   const bool c1 = C == 1 && conv_c1_tc_supported(k, Cout);
+  if (c1 && (int64_t)N * c.Ho * c.Wo > (1ll << 30)) {
+    set_error("conv2d: one input channel and more than 2^30 output pixels");
+    return DDPPO_E_CONFIG;
+  }
   if (!c1 && !gemm_conv_supported(c, x)) {
     set_error("conv2d: shape not covered by the implicit-im2col path");
     return DDPPO_E_CONFIG;
