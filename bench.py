@@ -110,9 +110,9 @@ class ClockSampler:
 
 # DRAM traffic of the update's contractions over their algorithmic bytes, from one ncu
 # capture of the same step at T = 16 (dram__bytes_read.sum + dram__bytes_write.sum over the
-# update's contraction launches: 10,400 MB against 15,690 MB algorithmic); the full-size
+# update's contraction launches: 9,264 MB against 13,336 MB algorithmic); the full-size
 # traffic is reported as this fraction of the live algorithmic bytes
-GEMM_TRAFFIC_OVER_ALGORITHMIC = 10400.0 / 15690.0
+GEMM_TRAFFIC_OVER_ALGORITHMIC = 9264.0 / 13336.0
 
 
 def _dist():

@@ -431,8 +431,9 @@ def ddppo_update_graph(h, on: bool = True) -> None:
 
 
 def ddppo_lstm_whole_segment(h, mode: int = 1) -> None:
-    """LSTM recurrence mode: 0 step by step (the default), 1 whole segment on CUDA cores,
-    2 tcgen05 forward; a bool selects 1 (True) or 0 (False)."""
+    """LSTM recurrence mode: 0 (the default) a cluster launch per layer and direction where the
+    shape is covered, else step by step, 1 whole segment on CUDA cores, 2 tcgen05 forward; a
+    bool selects 1 (True) or 0 (False)."""
     _check(lib().ddppo_lstm_whole_segment(h, int(mode)))
 
 

@@ -16,10 +16,10 @@
 //
 // Six CTAs (forward) or six building groups (gradient) an SM hide one another's build, MMA and
 // epilogue. Every wait is bounded.
-// Bound: HBM -- the fp32 output (2.1 GB for 4096 images of 128x128 into 32 channels), or dz.
-// With the patch matrix (1.9 GB) written by one kernel (827 us) and read by the GEMM the
-// encoder's pass took 19.8 ms there; now 16.9, with 458 us forward (5.0 TB/s) and 412 for
-// the gradient (bound by building the patches, 131,072 tiles of 128).
+// Bound: building the patches -- the shared-memory data pipe is 77% (forward) and 78% (gradient)
+// busy with their words and rows, HBM 51% and 36% (912 images of 128x128 into 32 channels). With
+// the patch matrix (1.9 GB for 4096 images) written by one kernel (827 us) and read by the GEMM
+// the encoder's pass took 19.5 ms; with this 16.7: 458 us forward, 412 the gradient.
 #include <algorithm>
 
 #include "gemm.cuh"

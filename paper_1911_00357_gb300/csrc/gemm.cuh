@@ -106,8 +106,6 @@ bool gemm_conv_supported(const ConvShape& c, const void* input);
 bool conv_wgrad_halo_ok(const ConvShape& c, const void* x, const void* dz);
 int conv_wgrad_halo(const ConvShape& c, const void* x, const void* dz, float* dw, int ldw, float beta,
                     const GemmWorkspace& ws, cudaStream_t s);
-// weight gradient of a 3x3 / stride-1 / pad-1 convolution, 64 -> 64 channels or multiples of
-// 128, every tap a shifted view of one staged box (wgrad_rows.cu); same result layout
 // the 7x7 / stride-2 single-channel stem (conv_stem.cu): forward into y [pixels, Cout], and
 // weight gradient into dw [Cout, ldw], 49 <= ldw <= 64 (zero past the 49th tap)
 bool conv_stem_ok(const ConvShape& c, const void* x);
@@ -116,6 +114,9 @@ int conv_stem(const ConvShape& c, const void* x, const void* w, int ldw, float* 
 bool conv_wgrad_stem_ok(const ConvShape& c, const void* x, const void* dz, const GemmWorkspace& ws);
 int conv_wgrad_stem(const ConvShape& c, const void* x, const void* dz, float* dw, int ldw, float beta,
                     const GemmWorkspace& ws, cudaStream_t s);
+// weight gradient of a 3x3 / stride-1 / pad-1 convolution, 64 -> 64 channels or multiples of
+// 128, every tap a shifted view of one staged box (wgrad_rows.cu); result laid out as
+// conv_wgrad_halo's
 bool conv_wgrad_rows_ok(const ConvShape& c, const void* x, const void* dz, const GemmWorkspace& ws);
 int conv_wgrad_rows(const ConvShape& c, const void* x, const void* dz, float* dw, int ldw, float beta,
                     const GemmWorkspace& ws, cudaStream_t s);

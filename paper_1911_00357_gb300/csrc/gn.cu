@@ -512,14 +512,15 @@ __global__ void __launch_bounds__(kThreads, CTAS) gn_image_kernel(GNApply a, Pix
   if (a.out_f8) block_amax(f8m, a.f8_amax);
 }
 
-// ---- backward reductions: g = dy (masked by relu_y > 0), xhat = (z - mu) rstd;
-//      per image and channel sum(g) and sum(g xhat); group means of gamma-weighted sums ----
+// the instance for the inputs that are present
 template <int V, int CTAS>
 void (*image_kernel(const GNApply& a))(GNApply, PixelCount, int, float) {
   if (a.resid) return a.zd ? gn_image_kernel<V, true, true, CTAS> : gn_image_kernel<V, true, false, CTAS>;
   return a.zd ? gn_image_kernel<V, false, true, CTAS> : gn_image_kernel<V, false, false, CTAS>;
 }
 
+// ---- backward reductions: g = dy (masked by the ReLU that followed), xhat = (z - mu) rstd;
+//      per image and channel sum(g) and sum(g xhat); group means of gamma-weighted sums ----
 template <int V>
 __global__ void __launch_bounds__(kThreads) gn_bwd_reduce_kernel(GNBack b, int HW, int C, int S,
                                                                  float* __restrict__ part,
@@ -841,7 +842,8 @@ __global__ void __launch_bounds__(kThreads) gn_bwd_slice_kernel(GNBack b, int HW
 // again. Here two blocks per SM take images in turn. One warp copies units (z, dy and the mask
 // bits of kRingRows P pixels, up to 16.5 KB) into a ring with bulk copies, an image's units for
 // the sums and then the same again for the gradient; eight warps consume them. The images
-// in work (2 x 152) stay in L2, and copies are in flight whatever the consumers wait for.
+// in work (2 x 152) stay in L2 -- 912 images of 1024 x 32 read 260 MB from memory, 239 MB of z
+// and dy once -- and copies are in flight whatever the consumers wait for.
 // Sums in the one-block-per-image order: bit-identical.
 // Measured on the encoder's 21 launches over 4096 frames: 4.14 ms, against 5.2 ms with one
 // block per image and the same masks (6.3 ms when the masks were read from the stored fp32

@@ -3,7 +3,7 @@
 // Some callers cannot allocate device memory where they need the loss: code that runs
 // while a stream is being captured into a CUDA graph in a capture mode that forbids
 // cudaMalloc, or a process whose device memory all belongs to another allocator. The
-// stateless ddppo_ppo_loss needs no scratch but reduces with a single thread block; this
+// stateless ddppo_ppo_loss needs no scratch but runs in a single thread-block cluster; this
 // variant spreads the samples over one block per 256 and keeps the per-block partial
 // sums in a library-owned array declared below, so it needs neither an allocation nor a
 // worker context.

@@ -285,8 +285,9 @@ static int reduce_blocks(size_t n) {
 // ---- the optimizer step ----
 // Both kernels walk the parameters four at a time, 16-byte accesses where the gradient
 // allows them (the other arrays are the library's). The update moves 28 bytes a parameter:
-// 8.5 M parameters (237 MB, above L2) take 32 us; with scalar accesses and the bias
-// corrections' two double-precision powers in every block it took 84 us.
+// 8.5 M parameters (237 MB) take 34 us, in which 176 MB pass through memory -- the last of what
+// it writes is still in L2 when it ends; with scalar accesses and the bias corrections' two
+// double-precision powers in every block it took 84 us.
 __device__ __forceinline__ float4 ld4(const float* p, bool aligned) {
   if (aligned) return *reinterpret_cast<const float4*>(p);
   return make_float4(p[0], p[1], p[2], p[3]);

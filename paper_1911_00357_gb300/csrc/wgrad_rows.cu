@@ -28,8 +28,9 @@
 // which 0 x makes a NaN. The second kernel therefore forms a sum that is not finite again, from
 // the pixels of its own tap alone.
 //
-// Measured (4096 images): 16x16, 64 -> 64 channels 106 us against 367 us for the gather form
-// (0.73 PFLOP/s; N = 64 leaves the MMAs bound by shared-memory reads); the seven
+// Measured (4096 images): 16x16, 64 -> 64 channels 97 us against 367 us for the gather form
+// (0.73 PFLOP/s; the tensor pipe is taken 77% of the time but computes 51%: MMAs of N = 64 wait
+// for their operands' shared-memory reads; x and dz come from memory once, 269 MB); the seven
 // convolutions of stages 3, 4 and the compression layer 72 us each on average, reduction
 // included. The encoder's ten such gradients: 0.80 ms against 2.9 ms.
 #include <algorithm>

@@ -26,8 +26,9 @@ Algorithmic bytes per unit (each operand read once, each result written once):
               prepared (untimed) before each timed step, as in the collect loop
 
   lstm        the 2-layer 512 LSTM forward over T = 128 steps of 32 envs (one update
-              minibatch of the ResNet workload, BF16) in each recurrence mode: 0 step by
-              step, 1 whole segment on CUDA cores, 2 whole segment on tcgen05 (times only)
+              minibatch of the ResNet workload, BF16) in each recurrence mode: 0 a cluster
+              launch per layer, 1 whole segment on CUDA cores, 2 whole segment on tcgen05
+              (times only)
 
     python -m paper_1911_00357_gb300.kernel_bench --only lstm group_norm
 

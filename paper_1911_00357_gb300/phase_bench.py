@@ -28,8 +28,9 @@ def main():
     ap.add_argument("--seed", type=int, default=3)
     ap.add_argument("--precision", type=int, default=None, help="override the preset's precision")
     ap.add_argument("--lstm-mode", type=int, default=0, choices=[0, 1, 2],
-                    help="LSTM recurrence: 0 step by step (default), 1 whole segment on CUDA "
-                         "cores, 2 tcgen05 forward")
+                    help="LSTM recurrence: 0 (default) a cluster launch per layer and direction "
+                         "where covered, else step by step, 1 whole segment on CUDA cores, "
+                         "2 tcgen05 forward")
     ap.add_argument("--gn-two-launch", action="store_true",
                     help="GroupNorm statistics and normalisation as two launches")
     ap.add_argument("--no-launch-overlap", action="store_true",
