@@ -780,8 +780,19 @@ __global__ void __launch_bounds__(TC_PTHREADS, 2)
 }
 
 // ---------------------------------------------------------------- host side
+// The encoder asks for a current context, which a host thread has only once a runtime call has
+// bound one: where it fails, the thread's device is bound and the map encoded again.
+static PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
+static CUresult CUDAAPI encode_bound(CUtensorMap* m, CUtensorMapDataType type, cuuint32_t rank, void* p,
+                                     const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
+                                     const cuuint32_t* estr, CUtensorMapInterleave il, CUtensorMapSwizzle sw,
+                                     CUtensorMapL2promotion l2, CUtensorMapFloatOOBfill fill) {
+  const CUresult r = g_encode(m, type, rank, p, dims, strides, box, estr, il, sw, l2, fill);
+  int dev = 0;
+  if (r == CUDA_SUCCESS || cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return r;
+  return g_encode(m, type, rank, p, dims, strides, box, estr, il, sw, l2, fill);
+}
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   static std::once_flag once;
   std::call_once(once, [] {
     void* p = nullptr;
@@ -789,9 +800,9 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
                                          &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
+      g_encode = (PFN_cuTensorMapEncodeTiled_v12000)p;
   });
-  return fn;
+  return g_encode ? encode_bound : nullptr;
 }
 
 // 2-D bf16 tensor [rows, cols] with row stride ld elements, box [box_rows, 64 columns]
