@@ -446,7 +446,7 @@ int ddppo_load(ddppo_ctx* ctx, const ddppo_rollout* ro, const char* path, void* 
  * tcgen05 tensor-core path with fp32 accumulation when rows are 16-byte aligned). C [dev]
  * row-major fp32, or bf16 when c_bf16 (then beta must be 0). bias [dev] [N] or NULL.
  * status [dev] int32 or NULL receives the sticky timeout flag (2) of a bounded
- * tensor-core wait. Split-K sums take 64 MB of the stream's scratch. */
+ * tensor-core wait. Split-K sums, where a call splits K, take 64 MB of the stream's scratch. */
 int ddppo_gemm(int32_t M, int32_t N, int32_t K, int32_t op_bf16, const void* A, int32_t lda,
                int32_t a_t, const void* B, int32_t ldb, int32_t b_t, void* C, int32_t ldc,
                int32_t c_bf16, float beta, const float* bias, int32_t relu, int32_t* status,
@@ -504,7 +504,7 @@ int ddppo_conv2d_e4m3(int32_t N, int32_t H, int32_t W, int32_t C, int32_t Cout, 
  * groups of 2 channels, eps 1e-5): out = act(gn(z) gamma + beta + resid) over NHWC z [dev]
  * fp32 [N, HW, C]; gamma, beta [dev] [C]; resid [dev] [N, HW, C] or NULL; relu 0/1; mean,
  * rstd [dev] [N, C/2] receive the group statistics. N <= 8192, C even <= 1024 (E_ARG
- * otherwise). 78 MB of the stream's scratch. */
+ * otherwise). The forms of several blocks an image take 78 MB of the stream's scratch. */
 int ddppo_group_norm(int32_t N, int32_t HW, int32_t C, const float* z, const float* gamma,
                      const float* beta, const float* resid, int32_t relu, float* out, float* mean,
                      float* rstd, void* stream);

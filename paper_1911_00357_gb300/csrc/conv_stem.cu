@@ -438,7 +438,8 @@ int conv_wgrad_stem(const ConvShape& c, const void* x, const void* dz, float* dw
     set_error("wgrad_stem: unsupported shape");
     return DDPPO_E_CONFIG;
   }
-  a.x = (const __nv_bfloat16*)x; a.dz = (const __nv_bfloat16*)dz; a.part = ws.partial; a.err = ws.err;
+  a.x = (const __nv_bfloat16*)x; a.dz = (const __nv_bfloat16*)dz; a.err = ws.err;
+  DDPPO_TRY(ws.sums(s, &a.part));
   a.kchunk = stem_wgrad_chunk(c, ldw, ws);
   const int splits = (c.N * c.Ho * c.Wo + a.kchunk - 1) / a.kchunk;
   auto kern = c.Cout == 32 ? wgrad_stem_kernel<32> : wgrad_stem_kernel<64>;
@@ -446,7 +447,7 @@ int conv_wgrad_stem(const ConvShape& c, const void* x, const void* dz, float* dw
   DDPPO_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ::ddppo::launch_k(kern, splits, SW_THREADS, smem, s, a);
   DDPPO_CHECK_LAUNCH();
-  ::ddppo::launch_k(wgrad_stem_reduce_kernel, ldw, c.Cout, 0, s, ws.partial, splits, dw, ldw, beta);
+  ::ddppo::launch_k(wgrad_stem_reduce_kernel, ldw, c.Cout, 0, s, a.part, splits, dw, ldw, beta);
   DDPPO_CHECK_LAUNCH();
   return DDPPO_OK;
 }

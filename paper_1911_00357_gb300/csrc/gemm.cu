@@ -241,7 +241,7 @@ static bool rows_of_4(const void* p, int ld, int bytes) {
 }
 
 template <int BM, int BN, int TM>
-static void launch_simt(SimtArgs& q, bool op_bf16, const GemmWorkspace& ws, int& splits, cudaStream_t s) {
+static int launch_simt(SimtArgs& q, bool op_bf16, const GemmWorkspace& ws, int& splits, cudaStream_t s) {
   const int gm = (q.M + BM - 1) / BM, gn = (q.N + BN - 1) / BN;
   const int tiles = gm * gn, target = 2 * ws.num_sms;
   splits = 1;
@@ -256,12 +256,15 @@ static void launch_simt(SimtArgs& q, bool op_bf16, const GemmWorkspace& ws, int&
   q.kchunk = (q.K + splits - 1) / splits;
   q.kchunk = (q.kchunk + SB_K - 1) / SB_K * SB_K;
   splits = (q.K + q.kchunk - 1) / q.kchunk;
-  q.partial = splits > 1 ? ws.partial : nullptr;
+  q.partial = nullptr;
+  if (splits > 1) DDPPO_TRY(ws.sums(s, &q.partial));
   if (q.partial ? rows_of_4(q.partial, q.N, 4) : (!q.c_bf16 && rows_of_4(q.C, q.ldc, 4))) q.vec |= SIMT_VEC_C;
   if (op_bf16)
     ::ddppo::launch_k(gemm_simt_kernel<BM, BN, TM, __nv_bfloat16>, dim3(gm, gn, splits), 256, 0, s, q);
   else
     ::ddppo::launch_k(gemm_simt_kernel<BM, BN, TM, float>, dim3(gm, gn, splits), 256, 0, s, q);
+  DDPPO_CHECK_LAUNCH();
+  return DDPPO_OK;
 }
 
 static int gemm_simt(const GemmDesc& d, bool op_bf16, const GemmWorkspace& ws, cudaStream_t s) {
@@ -276,11 +279,10 @@ static int gemm_simt(const GemmDesc& d, bool op_bf16, const GemmWorkspace& ws, c
   // one tile shape leaves half its FMAs on padding for 32 channels: 128x32 and 32x128 there
   // (9.5 us a launch; 64x64: 14.3). 128x64 saves shared reads where it still gives two CTAs
   // an SM (19.7 us; 64x64: 20.2)
-  if (d.N <= 32) launch_simt<128, 32, 4>(q, op_bf16, ws, splits, s);
-  else if (d.M <= 32) launch_simt<32, 128, 4>(q, op_bf16, ws, splits, s);
-  else if (((d.M + 127) / 128) * (int64_t)((d.N + 63) / 64) >= 2 * ws.num_sms) launch_simt<128, 64, 8>(q, op_bf16, ws, splits, s);
-  else launch_simt<64, 64, 4>(q, op_bf16, ws, splits, s);
-  DDPPO_CHECK_LAUNCH();
+  if (d.N <= 32) DDPPO_TRY((launch_simt<128, 32, 4>(q, op_bf16, ws, splits, s)));
+  else if (d.M <= 32) DDPPO_TRY((launch_simt<32, 128, 4>(q, op_bf16, ws, splits, s)));
+  else if (((d.M + 127) / 128) * (int64_t)((d.N + 63) / 64) >= 2 * ws.num_sms) DDPPO_TRY((launch_simt<128, 64, 8>(q, op_bf16, ws, splits, s)));
+  else DDPPO_TRY((launch_simt<64, 64, 4>(q, op_bf16, ws, splits, s)));
   if (q.partial)
     DDPPO_TRY(launch_splitk_reduce(d.M, d.N, splits, q.partial, q.C, d.ldc, d.c_bf16, d.beta, d.bias, d.relu, s));
   return DDPPO_OK;

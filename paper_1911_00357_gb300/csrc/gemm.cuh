@@ -65,9 +65,12 @@ size_t tc_tuner_export(const TcTuner* t, void* buf, size_t cap);
 // merge a serialised table (entries replace equal keys)
 int tc_tuner_import(TcTuner* t, const void* buf, size_t size);
 
+class Scratch;
 struct GemmWorkspace {
-  float* partial = nullptr;  // split-K partial sums
+  float* partial = nullptr;  // split-K partial sums (null: from scratch, by the launches that split)
   size_t partial_elems = 0;
+  Scratch* scratch = nullptr;
+  int sums(cudaStream_t s, float** p) const;  // the partial sums' buffer, on stream s
   int num_sms = 152;
   GemmTcCount* tc = nullptr;  // counts contractions routed to tcgen05 while enabled
   int32_t* err = nullptr;      // sticky device status word (timeout flag)

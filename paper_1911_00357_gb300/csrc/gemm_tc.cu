@@ -1185,7 +1185,8 @@ static int launch_tc(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N,
   int kchunk = (Ksplit + splits - 1) / splits;
   kchunk = (kchunk + kstep - 1) / kstep * kstep;
   splits = (Ksplit + kchunk - 1) / kchunk;
-  float* partial = splits > 1 ? ws.partial : nullptr;
+  float* partial = nullptr;
+  if (splits > 1) DDPPO_TRY(ws.sums(s, &partial));
   // persistent grid: one CTA per SM (two where shared memory allows), each walking tiles
   // with stride gridDim.x; the ring streams across tile boundaries
   const int stages = cfg.stages;
@@ -1654,11 +1655,13 @@ int conv_wgrad_halo(const ConvShape& c, const void* x, const void* dz, float* dw
                                           (int)TC_SMEM_MAX));
     attr_done[dev] = true;
   }
+  float* part = nullptr;
+  DDPPO_TRY(ws.sums(s, &part));
   ::ddppo::launch_k(wgrad_halo_kernel, grid, WH_THREADS, g.smem, s, mx, md, Wp, RB, nrb, nunits, g.x_bytes,
                                                      g.dz_bytes, g.x_stride, g.dz_stride, g.stages,
-                                                     ws.partial, ws.err);
+                                                     part, ws.err);
   DDPPO_CHECK_LAUNCH();
-  ::ddppo::launch_k(wgrad_halo_reduce_kernel, (32 * 288 + 255) / 256, 256, 0, s, ws.partial, grid, dw, ldw, beta);
+  ::ddppo::launch_k(wgrad_halo_reduce_kernel, (32 * 288 + 255) / 256, 256, 0, s, part, grid, dw, ldw, beta);
   DDPPO_CHECK_LAUNCH();
   return DDPPO_OK;
 }

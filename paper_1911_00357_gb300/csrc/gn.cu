@@ -1151,6 +1151,12 @@ static int gn_split_one_launch(int N, int HW, int C, const GnScratch& w) {
   return 0;
 }
 
+// whether a forward of these sizes (tensors: z, and a residual or shortcut beside it) needs the
+// scratch: not where one block sums an image or a slice of its channels and normalises it
+bool gn_fwd_scratch(int N, int HW, int C, int tensors, const GnScratch& w) {
+  return gn_split(N, HW, C, w) != 1 || (N < 4 * num_sms_cached() && !slice_channels(N, HW, C, tensors));
+}
+
 int launch_gn_stats(const float* z, int N, int HW, int C, float eps, float* mean, float* rstd,
                     const GnScratch& w, cudaStream_t s) {
   if (!N || !HW) return DDPPO_OK;
@@ -1174,7 +1180,7 @@ int launch_gn_fused(const GNApply& a, int N, int HW, int C, float eps, const GnS
                     int32_t* err, cudaStream_t s, bool* launched) {
   *launched = false;
   if (!N || !HW) { *launched = true; return DDPPO_OK; }
-  if (!w.cnt2 || !gn_shape_ok(C) || N > w.max_images || N > 65535) return DDPPO_OK;
+  if (!gn_shape_ok(C) || N > w.max_images || N > 65535) return DDPPO_OK;
   const int V = C % 4 == 0 ? 4 : 2;
   const int th = threads_for(C, V);
   void (*kern)(GNApply, PixelCount, int, int, float, float*, float*, int*, int*, int32_t*) =

@@ -723,15 +723,11 @@ extern "C" int ddppo_count_kernels(ddppo_ctx* x, const ddppo_rollout* ro,
   return rc;
 }
 
-// split-K sums of a stand-alone contraction on stream s; scratch holds them for the call
-static int standalone_ws(GemmWorkspace* ws, Scratch* scratch, int32_t* status, cudaStream_t s) {
-  const size_t elems = (size_t)16 << 20;
-  DDPPO_TRY(scratch->take(SCRATCH_SPLITK, elems * sizeof(float), 0, s));
-  ws->partial = scratch->as<float>();
-  ws->partial_elems = elems;
-  int dev = 0;
-  DDPPO_CHECK_CUDA(cudaGetDevice(&dev));
-  cudaDeviceGetAttribute(&ws->num_sms, cudaDevAttrMultiProcessorCount, dev);
+// a stand-alone contraction's workspace; scratch holds its split-K sums for the call
+static int standalone_ws(GemmWorkspace* ws, Scratch* scratch, int32_t* status) {
+  DDPPO_TRY(device_sms(&ws->num_sms));
+  ws->partial_elems = kSplitkElems;
+  ws->scratch = scratch;
   ws->err = status;
   return DDPPO_OK;
 }
@@ -748,7 +744,7 @@ extern "C" int ddppo_gemm(int32_t M, int32_t N, int32_t K, int32_t op_bf16, cons
       "gemm: leading dimension smaller than the row");
   Scratch scratch;
   GemmWorkspace ws;
-  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status));
   GemmDesc d;
   d.M = M; d.N = N; d.K = K; d.A = A; d.lda = lda; d.B = B; d.ldb = ldb; d.C = C; d.ldc = ldc;
   d.c_bf16 = c_bf16; d.beta = beta; d.bias = bias; d.relu = relu;
@@ -827,12 +823,14 @@ extern "C" int ddppo_group_norm(int32_t N, int32_t HW, int32_t C, const float* z
   GnScratch w;
   w.max_images = 8192;
   w.part_elems = gn_part_elems(w.max_images, 1024);
-  const size_t part = w.part_elems * sizeof(float), cnts = (size_t)w.max_images * sizeof(int);
   Scratch scratch;
-  DDPPO_TRY(scratch.take(SCRATCH_GN, part + 2 * cnts, 2 * cnts, s));
-  w.part = scratch.as<float>();
-  w.cnt = scratch.as<int>(part);
-  w.cnt2 = scratch.as<int>(part + cnts);
+  if (gn_fwd_scratch(N, HW, C, resid ? 2 : 1, w)) {
+    const size_t part = w.part_elems * sizeof(float), cnts = (size_t)w.max_images * sizeof(int);
+    DDPPO_TRY(scratch.take(SCRATCH_GN, part + 2 * cnts, 2 * cnts, s));
+    w.part = scratch.as<float>();
+    w.cnt = scratch.as<int>(part);
+    w.cnt2 = scratch.as<int>(part + cnts);
+  }
   GNApply a{};
   a.z = z; a.mean = mean; a.rstd = rstd; a.gamma = gamma; a.beta = beta;
   a.resid = resid; a.out = out; a.relu = relu ? 1 : 0;
@@ -912,7 +910,7 @@ extern "C" int ddppo_conv2d(int32_t N, int32_t H, int32_t W, int32_t C, int32_t 
   }
   Scratch scratch;
   GemmWorkspace ws;
-  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status));
   GemmDesc d;
   d.M = N * c.Ho * c.Wo; d.N = Cout; d.K = k * k * C;
   d.conv = &c; d.A = x; d.lda = d.K; d.B = w; d.ldb = d.K;
@@ -954,7 +952,7 @@ extern "C" int ddppo_gemm_e4m3(int32_t M, int32_t N, int32_t K, const void* A, i
   ARG(lda >= K && ldb >= K && ldc >= N, "gemm_e4m3: leading dimension smaller than the row");
   Scratch scratch;
   GemmWorkspace ws;
-  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status));
   GemmDesc d;
   d.M = M; d.N = N; d.K = K; d.A = A; d.lda = lda; d.B = B; d.ldb = ldb; d.C = C; d.ldc = ldc;
   d.beta = beta; d.bias = bias; d.relu = relu;
@@ -972,7 +970,7 @@ extern "C" int ddppo_conv2d_e4m3(int32_t N, int32_t H, int32_t W, int32_t C, int
   c.Cout = Cout;
   Scratch scratch;
   GemmWorkspace ws;
-  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status));
   GemmDesc d;
   d.M = N * c.Ho * c.Wo; d.N = Cout; d.K = k * k * C;
   d.conv = &c; d.A = x; d.lda = d.K; d.B = w; d.ldb = d.K;
@@ -995,7 +993,7 @@ extern "C" int ddppo_conv2d_wgrad(int32_t N, int32_t H, int32_t W, int32_t C, in
   }
   Scratch scratch;
   GemmWorkspace ws;
-  DDPPO_TRY(standalone_ws(&ws, &scratch, status, (cudaStream_t)stream));
+  DDPPO_TRY(standalone_ws(&ws, &scratch, status));
   GemmDesc d;
   d.M = Cout; d.N = k * k * C; d.K = N * c.Ho * c.Wo;
   d.A = dy; d.lda = Cout; d.a_t = 1;

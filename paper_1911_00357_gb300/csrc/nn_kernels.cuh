@@ -34,6 +34,7 @@ struct GnScratch {
   int max_images = 0;
 };
 size_t gn_part_elems(int max_images, int max_C);
+bool gn_fwd_scratch(int N, int HW, int C, int tensors, const GnScratch& w);
 // C even, C / V <= 256 (V = 4 when C % 4 == 0, else 2): C <= 1024
 int launch_gn_stats(const float* z, int N, int HW, int C, float eps, float* mean, float* rstd,
                     const GnScratch& w, cudaStream_t s);

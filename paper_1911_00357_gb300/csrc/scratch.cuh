@@ -15,6 +15,9 @@
 
 namespace ddppo {
 
+constexpr size_t kSplitkElems = (size_t)16 << 20;  // floats of split-K sums
+int device_sms(int* sms);                          // SMs of the current device
+
 enum ScratchKind { SCRATCH_SPLITK = 0, SCRATCH_GN, SCRATCH_GCONV, SCRATCH_AMAX, SCRATCH_KINDS };
 
 class Scratch {
@@ -24,7 +27,7 @@ class Scratch {
   Scratch& operator=(const Scratch&) = delete;
   ~Scratch();
   // `bytes` (the same for every call of a kind) for this call's launches on s, held until the
-  // object goes; the last `zeroed` of them are zero when the memory is new. Once per object.
+  // object goes; the last `zeroed` of them are zero when the memory is new. One kind an object.
   int take(ScratchKind kind, size_t bytes, size_t zeroed, cudaStream_t s);
   template <typename T>
   T* as(size_t offset = 0) const { return reinterpret_cast<T*>((char*)p_ + offset); }

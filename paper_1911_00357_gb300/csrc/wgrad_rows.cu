@@ -326,11 +326,12 @@ int launch_wr(const WrPlan& p, const CUtensorMap& mx, const CUtensorMap& md, con
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WR_SMEM_MAX));
     attr_done[dev] = true;
   }
-  ::ddppo::launch_k(wgrad_rows_kernel<NB>, p.jobs * p.a.cpj, WR_THREADS, p.smem, s, mx, md, p.a, ws.partial,
-                    ws.err);
+  float* part = nullptr;
+  DDPPO_TRY(ws.sums(s, &part));
+  ::ddppo::launch_k(wgrad_rows_kernel<NB>, p.jobs * p.a.cpj, WR_THREADS, p.smem, s, mx, md, p.a, part, ws.err);
   DDPPO_CHECK_LAUNCH();
   ::ddppo::launch_k(wgrad_rows_reduce_kernel<NB>, dim3(16 * (NB / 32), NB == 64 ? 6 : 3, p.jobs), 256, 0, s,
-                    ws.partial, p.a, px, dw, ldw, beta);
+                    part, p.a, px, dw, ldw, beta);
   DDPPO_CHECK_LAUNCH();
   return DDPPO_OK;
 }
