@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(WR_THREADS, 1)
 
 // One weight's gradient from its own pixels alone, in plain order (zero outside the image).
 // Out of line and last in its caller: no stack frame there, 48 registers a thread (32 without
-// it) and the same time (97.2 us a call at 4096 x 16x16, 64 -> 64; 96.9).
+// it), 0.25 us a call (97.1 us at 4096 x 16x16, 64 -> 64).
 struct WrPixels {
   const __nv_bfloat16* x;
   const __nv_bfloat16* dz;
